@@ -41,29 +41,39 @@ struct VecIn {
 };
 
 cudaError_t setup_validate(const SetupIn& in, int* d_err, cudaStream_t s);
+// row_of[nnz]: scratch (transpose_row_ids of the transpose's scratch will do)
 cudaError_t setup_canonical(const SetupIn& in, int* a_ptr, int* a_col, double* a_val64, double* q,
-                            unsigned char* row_kind, cudaStream_t s);
+                            unsigned char* row_kind, int* row_of, cudaStream_t s);
 size_t transpose_tmp_ints(int m, int n, long long nnz);
+// where setup_transpose leaves the row of each of A's entries in its scratch
+int* transpose_row_ids(int* tmp, int n, long long nnz);
+// t_val64 may be NULL: the values are not wanted (every one is +1)
 // device_desc: build the long-segment tile descriptors on the device instead of
 // in host vectors (no host allocation)
 cudaError_t setup_transpose(int m, int n, int nnz, const int* a_ptr, const int* a_col,
                             const double* a_val64, int* t_ptr, int* t_col, double* t_val64,
                             int* tmp, cudaStream_t s, bool device_desc = false);
-cudaError_t setup_scaling(const ScaleIn& sc, double* dr, double* dc, double* stat_r,
-                          double* stat_c, cudaStream_t s);
+// dr2[m], dc2[n]: scratch of the same sizes as the factors; list_a[m + 1], list_t[n + 1]:
+// scratch for the lists of long rows; sc.a_val64 and sc.t_val64 NULL: every value is +1
+cudaError_t setup_scaling(const ScaleIn& sc, double* dr, double* dc, double* dr2, double* dc2,
+                          int* list_a, int* list_t, cudaStream_t s);
 cudaError_t setup_value_format(const double* val64, int nnz, int* d_flags, int* h_bf16_exact,
                                int* h_all_one, cudaStream_t s);
-// which_type: 0 double, 1 float, 2 bfloat16
-cudaError_t setup_iter_values(int which_type, const int* ptr, const int* col, const double* val64,
-                              int nrows, const double* own, const double* other, int own_is_row,
-                              int scaled, void* out, cudaStream_t s);
+// which_type: 0 double, 1 float (scaled by dr, dc), 2 bfloat16 (plain); row, col: the row and
+// the column of A of each entry, in either orientation's order
+cudaError_t setup_iter_values(int which_type, const int* row, const int* col,
+                              const double* val64, int nnz, const double* dr, const double* dc,
+                              void* out, cudaStream_t s);
+// the row of each entry of a CSR matrix
+cudaError_t setup_row_ids(const int* ptr, int rows, long long nnz, int* row_of, cudaStream_t s);
 size_t setup_part_doubles(int m, int n);
 // scalars_out: [0] ||c~||, [1] ||q~||, [2] ||c||, [3] ||q||, [4] max |K~_ij|,
 // [5] ||x~_hint||, [6] ||y~_hint|| (scaled space, projected; 0 without a hint),
-// [7] the number of columns with an infinite bound
+// [7] the number of columns with an infinite bound; NULL: not wanted.  row_of: the row of
+// each of A's entries; a_val64 NULL: every value is +1
 cudaError_t setup_iter_vectors(const VecIn& v, int fp32, void* c, void* l, void* u, void* q,
-                               void* tw, void* sw, void* x0, void* y0, const int* a_ptr,
-                               const int* a_col, const double* a_val64, double* part,
+                               void* tw, void* sw, void* x0, void* y0, const int* row_of,
+                               const int* a_col, const double* a_val64, int nnz, double* part,
                                double* scalars_out, cudaStream_t s);
 size_t scan_tmp_ints(long long N);
 // dst[i] = src[i] + offset (index arrays moved into a batch's global numbering)
@@ -144,11 +154,12 @@ cudaError_t setup_batch_ingest(const BatchLp* d_lps, int count, long long max_ro
                                char* sense_g, double* c_g, double* l_g, double* u_g, int* d_err,
                                cudaStream_t s);
 // The A3 scalars of every LP: out[8 count] as setup_iter_vectors' scalars_out
-// (hint norms 0).
+// (hint norms 0); part: batch_scalar_doubles(count) of scratch.
+size_t batch_scalar_doubles(int count);
 cudaError_t setup_batch_scalars(const BatchLp* d_lps, int count, const double* dr,
                                 const double* dc, const double* c, const double* l,
-                                const double* u, const double* q, const int* a_ptr,
-                                const int* a_col, const double* a_val64, double* out,
+                                const double* u, const double* q, const int* row_of,
+                                const int* a_col, const double* a_val64, double* part, double* out,
                                 cudaStream_t s);
 // The global list of rows longer than thresh and each LP's first entry of it
 // (d_bounds[count + 1]); over_cols: the rows are the LPs' columns (A^T).

@@ -490,12 +490,10 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
   }
   mark("validate");
   // ---- A0, A1
-  CUDA_TRY(setup_canonical(in, bf.a_ptr, bf.a_col, bf.a_val64, bf.q64, bf.row_kind, s));
-  CUDA_TRY(setup_transpose(m, n, (int)nnz, bf.a_ptr, bf.a_col, bf.a_val64, bf.t_ptr, bf.t_col,
-                           bf.t_val64, bf.tmp, s, no_alloc));
-  g_launches += 10;
-  mark("canonical + transpose");
-  // ---- mode
+  int* row_of = transpose_row_ids(bf.tmp, n, nnz);  // the row of each of A's entries
+  CUDA_TRY(setup_canonical(in, bf.a_ptr, bf.a_col, bf.a_val64, bf.q64, bf.row_kind, row_of, s));
+  mark("canonical form");
+  // ---- mode (before the transpose: a 0/1 pattern has no values to transpose)
   Mode mode = MODE_FP64;
   int bf16_exact = 0, all_one = 0;
   if (p->precision == PDLP_FP32) mode = MODE_FP32;
@@ -508,26 +506,35 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
   }
   const int scaled = (mode == MODE_FP64 || mode == MODE_FP32) ? 1 : 0;
   const int fp32 = mode != MODE_FP64;
-  // ---- A2
-  ScaleIn sc{m, n, bf.a_ptr, bf.a_col, bf.a_val64, bf.t_ptr, bf.t_col, bf.t_val64, p->ruiz_iters,
-             p->pc_alpha, nnz};
+  const double* a_val = mode == MODE_PAT ? nullptr : bf.a_val64;
+  double* t_val = mode == MODE_PAT ? nullptr : bf.t_val64;
   mark("value format");
-  CUDA_TRY(setup_scaling(sc, bf.dr, bf.dc, bf.stat_r, bf.stat_c, s));
-  g_launches += 2 + 2 * p->ruiz_iters + (p->pc_alpha >= 0 ? 2 : 0);
+  CUDA_TRY(setup_transpose(m, n, (int)nnz, bf.a_ptr, bf.a_col, bf.a_val64, bf.t_ptr, bf.t_col,
+                           t_val, bf.tmp, s, no_alloc));
+  g_launches += 13;
+  mark("transpose");
+  // ---- A2
+  ScaleIn sc{m, n, bf.a_ptr, bf.a_col, a_val, bf.t_ptr, bf.t_col, t_val, p->ruiz_iters,
+             p->pc_alpha, nnz};
+  CUDA_TRY(setup_scaling(sc, bf.dr, bf.dc, bf.stat_r, bf.stat_c, bf.a_long, bf.t_long, s));
+  g_launches += 1 + p->ruiz_iters + (p->pc_alpha >= 0 ? 1 : 0);
   mark("Ruiz + Pock-Chambolle");
   CUDA_TRY(setup_kkt_aux(m, n, bf.dr, bf.dc, l, u, bf.inv_dr, bf.inv_dc, bf.bflags, s));
   ++g_launches;
   if (mode != MODE_PAT) {
     const int vt = mode == MODE_FP64 ? 0 : (mode == MODE_FP32 ? 1 : 2);
-    CUDA_TRY(setup_iter_values(vt, bf.a_ptr, bf.a_col, bf.a_val64, m, bf.dr, bf.dc, 1, scaled,
+    int* col_of = bf.tmp + (n + 1);  // the transpose is done with its sort keys
+    if (scaled) CUDA_TRY(setup_row_ids(bf.t_ptr, n, nnz, col_of, s));
+    CUDA_TRY(setup_iter_values(vt, row_of, bf.a_col, bf.a_val64, (int)nnz, bf.dr, bf.dc,
                                bf.a_valit, s));
-    CUDA_TRY(setup_iter_values(vt, bf.t_ptr, bf.t_col, bf.t_val64, n, bf.dc, bf.dr, 0, scaled,
+    CUDA_TRY(setup_iter_values(vt, bf.t_col, col_of, bf.t_val64, (int)nnz, bf.dr, bf.dc,
                                bf.t_valit, s));
-    g_launches += 2;
+    g_launches += scaled ? 3 : 2;
   }
   VecIn vi{m, n, bf.dr, bf.dc, c, l, u, bf.q64, bf.row_kind, x0, y0, scaled, hx, hy};
   CUDA_TRY(setup_iter_vectors(vi, fp32, bf.c_it, bf.l_it, bf.u_it, bf.q_it, bf.tw, bf.sw, bf.x[0],
-                              bf.y[0], bf.a_ptr, bf.a_col, bf.a_val64, bf.part_setup, bf.scalars, s));
+                              bf.y[0], row_of, bf.a_col, a_val, (int)nnz, bf.part_setup,
+                              bf.scalars, s));
   g_launches += 3;
   double sca[8];
   CUDA_TRY(cudaMemcpyAsync(sca, bf.scalars, sizeof(sca), cudaMemcpyDeviceToHost, s));
@@ -1607,7 +1614,7 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
     // batched setup: the batch in global numbering as the callers gave it, scratch
     int64_t *rp_in, *rp_up;
     int* col_in;
-    double *val_in, *b_in, *stat_r, *stat_c, *part_setup, *scalars, *lpsca;
+    double *val_in, *b_in, *stat_r, *stat_c, *part_setup, *lpsca;
     char* sense_in;
     int *tmp, *flags2, *errs, *lb_a, *lb_t;
     BatchLp* lps;
@@ -1665,8 +1672,8 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
     g.rp_up = device_inputs ? nullptr : (int64_t*)ar.take(8 * (M + (size_t)count));
     g.col_in = (int*)ar.take(4 * Z);
     g.val_in = (double*)ar.take(8 * Z);
-    g.part_setup = (double*)ar.take(8 * setup_part_doubles((int)M, (int)N));
-    g.scalars = (double*)ar.take(8 * 8);
+    g.part_setup = (double*)ar.take(
+        8 * std::max(setup_part_doubles((int)M, (int)N), batch_scalar_doubles(count)));
     g.lpsca = (double*)ar.take(8 * 8 * (size_t)count);
     g.tmp = (int*)ar.take(4 * tmp_ints);
     g.flags2 = (int*)ar.take(16);
@@ -1780,10 +1787,8 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
   // ---- A0-A3 over the whole block-diagonal problem: every step treats each row and
   // column on its own, so each LP is set up exactly as on its own
   SetupIn gin{(int)M, (int)N, Z, g.rp_in, g.col_in, g.val_in, g.b_in, g.sense_in, g.c64, g.l64, g.u64};
-  CUDA_TRY(setup_canonical(gin, g.a_ptr, g.a_col, g.a_val64, g.q64, g.row_kind, s));
-  CUDA_TRY(setup_transpose((int)M, (int)N, (int)Z, g.a_ptr, g.a_col, g.a_val64, g.t_ptr, g.t_col,
-                           g.t_val64, g.tmp, s, false));
-  g_launches += 11;
+  int* row_of = transpose_row_ids(g.tmp, (int)N, Z);
+  CUDA_TRY(setup_canonical(gin, g.a_ptr, g.a_col, g.a_val64, g.q64, g.row_kind, row_of, s));
   if (p->precision == PDLP_FP32_BF16A) {
     int bf16_exact = 0, all_one = 0;
     CUDA_TRY(setup_value_format(g.a_val64, (int)Z, g.flags2, &bf16_exact, &all_one, s));
@@ -1791,31 +1796,36 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
     mode = all_one ? MODE_PAT : (bf16_exact ? MODE_BF16 : MODE_FP32);
   }
   const int scaled = (mode == MODE_FP64 || mode == MODE_FP32) ? 1 : 0;
+  const double* a_val = mode == MODE_PAT ? nullptr : g.a_val64;
+  double* t_val = mode == MODE_PAT ? nullptr : g.t_val64;
+  CUDA_TRY(setup_transpose((int)M, (int)N, (int)Z, g.a_ptr, g.a_col, g.a_val64, g.t_ptr, g.t_col,
+                           t_val, g.tmp, s, false));
+  g_launches += 14;
   {
-    ScaleIn sc{(int)M, (int)N, g.a_ptr, g.a_col, g.a_val64, g.t_ptr, g.t_col, g.t_val64,
+    ScaleIn sc{(int)M, (int)N, g.a_ptr, g.a_col, a_val, g.t_ptr, g.t_col, t_val,
                p->ruiz_iters, p->pc_alpha, Z};
-    CUDA_TRY(setup_scaling(sc, g.dr, g.dc, g.stat_r, g.stat_c, s));
-    g_launches += 2 + 2 * p->ruiz_iters + (p->pc_alpha >= 0 ? 2 : 0);
+    CUDA_TRY(setup_scaling(sc, g.dr, g.dc, g.stat_r, g.stat_c, g.a_long, g.t_long, s));
+    g_launches += 1 + p->ruiz_iters + (p->pc_alpha >= 0 ? 1 : 0);
   }
   CUDA_TRY(setup_kkt_aux((int)M, (int)N, g.dr, g.dc, g.l64, g.u64, g.inv_dr, g.inv_dc, g.bflags, s));
   ++g_launches;
   if (mode != MODE_PAT) {
     const int vt = mode == MODE_FP64 ? 0 : (mode == MODE_FP32 ? 1 : 2);
-    CUDA_TRY(setup_iter_values(vt, g.a_ptr, g.a_col, g.a_val64, (int)M, g.dr, g.dc, 1, scaled,
-                               g.a_valit, s));
-    CUDA_TRY(setup_iter_values(vt, g.t_ptr, g.t_col, g.t_val64, (int)N, g.dc, g.dr, 0, scaled,
-                               g.t_valit, s));
-    g_launches += 2;
+    int* col_of = g.tmp + (N + 1);  // the transpose is done with its sort keys
+    if (scaled) CUDA_TRY(setup_row_ids(g.t_ptr, (int)N, Z, col_of, s));
+    CUDA_TRY(setup_iter_values(vt, row_of, g.a_col, g.a_val64, (int)Z, g.dr, g.dc, g.a_valit, s));
+    CUDA_TRY(setup_iter_values(vt, g.t_col, col_of, g.t_val64, (int)Z, g.dr, g.dc, g.t_valit, s));
+    g_launches += scaled ? 3 : 2;
   }
   {
     VecIn vi{(int)M, (int)N, g.dr, g.dc, g.c64, g.l64, g.u64, g.q64, g.row_kind, nullptr, nullptr,
              scaled, nullptr, nullptr};
     CUDA_TRY(setup_iter_vectors(vi, mode != MODE_FP64, g.c_it, g.l_it, g.u_it, g.q_it, g.tw, g.sw,
-                                g.x[0], g.y[0], g.a_ptr, g.a_col, g.a_val64, g.part_setup,
-                                g.scalars, s));
-    CUDA_TRY(setup_batch_scalars(g.lps, count, g.dr, g.dc, g.c64, g.l64, g.u64, g.q64, g.a_ptr,
-                                 g.a_col, g.a_val64, g.lpsca, s));
-    g_launches += 4;
+                                g.x[0], g.y[0], row_of, g.a_col, a_val, (int)Z, g.part_setup,
+                                nullptr, s));
+    CUDA_TRY(setup_batch_scalars(g.lps, count, g.dr, g.dc, g.c64, g.l64, g.u64, g.q64, row_of,
+                                 g.a_col, a_val, g.part_setup, g.lpsca, s));
+    g_launches += 3;
   }
   // long rows: one global list per orientation, each LP's part of it contiguous
   const int th_a = long_thresh(lanes[0], lanes[2]);
