@@ -143,8 +143,11 @@ typedef struct {
                            (small LPs, such as the 200 x 400 relaxations: no launch per
                            attempt), which copies the LP into shared memory when it fits
                            and otherwise runs the cooperative kernel as one block; 0
-                           (default): two kernel launches per attempt.  Same iteration
-                           either way.  Batches: 1 runs one cooperative kernel per check
+                           (default): the library's choice -- for one LP with float32
+                           iterates that fits, one block or one cooperative kernel with the
+                           LP in the SMs' shared memory (unless lanes_A, lanes_AT, autotune,
+                           tiles or halpern ask for the launches), else two kernel launches
+                           per attempt.  Same iteration either way.  Batches: 1 runs one cooperative kernel per check
                            period over every LP of the batch (three grid barriers per
                            attempt); 2 is rejected. */
   int autotune;         /* 1: before iterating, time whole step attempts (primal kernel,
@@ -438,8 +441,8 @@ int pdlp_solve_device(const pdlp_csr* A, const double* b, const char* sense, con
  *       away without bound,
  *   [2] one whole attempt (the primal step, then the dual half-step),
  *   [3] the float64 KKT pass over A, [4] the float64 KKT pass over A^T,
- *   [5] one attempt inside the persistent step kernel (reps attempts in one
- *       launch; 0 when p->persistent is 0),
+ *   [5] one attempt inside the kernel that holds a whole check period (reps attempts
+ *       in one launch; 0 where the steps run as separate launches, persistent_form 0),
  *   [6] one whole KKT block as a check runs it (candidates, both passes, the
  *       decision, the restart, the flags; a reset of the check flag before each,
  *       so each block starts after a full dependency as in a solve; bytes: [3]

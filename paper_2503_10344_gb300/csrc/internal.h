@@ -59,6 +59,78 @@ inline SmemLayout smem_layout(long long m, long long n, long long nnz, int it, b
   return L;
 }
 
+// The resident step kernel (resident_kernels.cuh): one LP spread over the shared memory of G
+// blocks, one per SM.
+constexpr int kResBlock = 512;  // threads per block at most
+constexpr int kResLong = 64;     // rows longer than this are summed by a warp
+constexpr int kResGatherY = 8;   // gathers in flight per thread: entries of y,
+constexpr int kResGatherX = 4;   // pairs
+constexpr int kResBuckets = 2048;  // buckets the gathers are ordered into
+constexpr int kResReplicas = 16;   // copies of the posted words
+constexpr int kResPoll = 5;      // slots a lane reads at a time (152 SMs: one round)
+constexpr int kResMinStage = 2048;  // nonzeros of A staged at a time at least, if not all are
+
+// Byte offsets of a block's copy of its part of the LP: nt columns with zt nonzeros, na rows
+// with za.  vb: bytes of a matrix value (0: a 0/1 pattern); implicit: per-element step weights
+// are kept.  The stage follows at `bytes`.
+struct ResLayout {
+  int t_ptr, t_col, t_val, t_lng, a_ptr, a_col, a_val, a_lng;
+  int c, l, u, tw, q, sw, kind, x0, x1, y0, y1, sx, sy;
+  int bytes;
+};
+__host__ __device__ inline ResLayout res_layout(int nt, int zt, int na, int za, int vb,
+                                                bool implicit) {
+  ResLayout L;
+  long long o = 0;
+  auto take = [&o](long long b) -> int {
+    const long long r = o;
+    o += (b + 15) / 16 * 16;
+    return (int)(r < (1LL << 30) ? r : (1LL << 30));
+  };
+  L.t_ptr = take(4LL * (nt + 1));
+  L.t_col = take(4LL * zt);
+  L.t_val = take((long long)vb * zt);
+  L.t_lng = take(4LL * (zt / kResLong + 1));
+  L.a_ptr = take(4LL * (na + 1));
+  L.a_col = take(4LL * za);
+  L.a_val = take((long long)vb * za);
+  L.a_lng = take(4LL * (za / kResLong + 1));
+  L.c = take(4LL * nt);
+  L.l = take(4LL * nt);
+  L.u = take(4LL * nt);
+  L.tw = take(implicit ? 4LL * nt : 0);
+  L.q = take(4LL * na);
+  L.sw = take(implicit ? 4LL * na : 0);
+  L.kind = take(na);
+  L.x0 = take(4LL * nt);
+  L.x1 = take(4LL * nt);
+  L.y0 = take(4LL * na);
+  L.y1 = take(4LL * na);
+  L.sx = take(4LL * nt);
+  L.sy = take(4LL * na);
+  L.bytes = (int)(o < (1LL << 30) ? o : (1LL << 30));
+  return L;
+}
+
+// What the cuts come to (k_res_plan): the largest part of each side, the longest row, and the
+// largest block's bytes without the stage
+struct ResSizes {
+  int t_rows, t_nnz, a_rows, a_nnz, max_len, bytes;
+};
+
+struct ResPlan {
+  int G;                       // blocks (0: the kernel is not used)
+  const int *cut_t, *cut_a;    // [G + 1] first column / row of each block
+  ulonglong2* slot;            // [kResReplicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
+  ulonglong2* ex_x;            // [n] published (x', dx), tag
+  unsigned long long* ex_y[2]; // [m] published y, tag
+  int threads, smem;           // per block
+  int lanes_t, lanes_a;        // lanes per row of the sums over A^T and A
+  int bits_t, bits_a;          // bits of an index of a gather (the rest of its word: the place)
+  int shift_t, shift_a;        // index >> shift: the bucket it is ordered by
+  int cap_t, cap_a;            // nonzeros staged at a time
+};
+
 struct IterRaw {
   const int *a_ptr, *a_col;
   const void* a_val;
@@ -88,6 +160,7 @@ struct IterRaw {
   // that much shared memory; 0 runs the one-block k_persist from global memory
   SmemLayout smem;
   const int *ord_t, *ord_a;  // its order of the columns and rows (longest first)
+  ResPlan res;               // the resident form (res.G > 0)
   // Halpern variant (pdlp_params.halpern): its iterate and anchor (iterate type; NULL off)
   void *hx, *hy;
   const void *hax, *hay;
@@ -105,6 +178,11 @@ cudaError_t launch_persist_bf16(int lanes_a, int lanes_t, const IterRaw& r, int 
                                 int grid, int* grid_out, cudaStream_t s);
 cudaError_t launch_persist_pat(int lanes_a, int lanes_t, const IterRaw& r, int max_attempts,
                                int grid, int* grid_out, cudaStream_t s);
+
+// resident step kernel (float32 iterates): the step attempts of a check period
+cudaError_t launch_resident_fp32(const IterRaw& r, int max_attempts, cudaStream_t s);
+cudaError_t launch_resident_bf16(const IterRaw& r, int max_attempts, cudaStream_t s);
+cudaError_t launch_resident_pat(const IterRaw& r, int max_attempts, cudaStream_t s);
 
 // blocks of the tile kernels of a form (primal, dual) resident at once on this device
 cudaError_t tile_resident_fp32(int form, int* primal_blocks, int* dual_blocks);

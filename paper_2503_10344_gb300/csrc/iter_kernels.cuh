@@ -466,6 +466,14 @@ __device__ __forceinline__ void step_factors(const DevState* st, long long k, fl
   }
 }
 
+// whether the accepted iterations fill check periods (a 32-bit remainder where it will do: the
+// 64-bit one is a long chain in the deciding thread)
+__device__ __forceinline__ bool period_ends(const DevState* st) {
+  const unsigned long long it = (unsigned long long)st->iters;
+  return (it >> 32) == 0 ? (unsigned)it % (unsigned)st->period == 0
+                         : it % (unsigned long long)st->period == 0;
+}
+
 // A6: adaptive step-size rule, decided once per attempt by one thread, in the
 // iterate precision; fd, fi are the step-rule factors of this attempt
 // (k = attempts + 1), fetched by the caller ahead of time.  In the
@@ -506,7 +514,7 @@ __device__ __forceinline__ void decide_step(DevState* st, T dx2, T dy2, T dkd, T
     st->pw_f = (float)eta;
     st->sum_w += (double)eta;
     st->iters += 1;
-    if (st->iters % st->period == 0 || st->iters >= st->iter_limit) st->check_due = 1;
+    if (period_ends(st) || st->iters >= st->iter_limit) st->check_due = 1;
   } else {
     st->pending_w = 0.0;
     st->pw_f = 0.0f;

@@ -6,6 +6,7 @@
 
 #include "internal.h"
 #include "iter_kernels.cuh"
+#include "resident_kernels.cuh"
 #include "tile_kernels.cuh"
 #include "smem_kernels.cuh"
 #include "wtile_kernels.cuh"
@@ -178,6 +179,39 @@ cudaError_t launch_persist_la(int lanes_t, const IterData<T, V>& d, int max_atte
     case 32: return launch_persist_one<LA, 32, T, V, IMPLICIT>(d, max_attempts, grid, grid_out, s);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// The resident step kernel: one cooperative launch of r.res.G blocks, at most one per SM.
+// max_attempts = 0 launches nothing and answers whether a block fits on an SM.
+template <typename V, bool IMPLICIT>
+cudaError_t launch_resident_t(const IterRaw& r, int max_attempts, cudaStream_t s) {
+  const IterData<float, V> d = typed<float, V>(r);
+  auto kern = k_resident<V, IMPLICIT>;
+  // its dynamic shared memory: a property of the kernel on this device, so every launch sets
+  // the same value, the largest (a launch of another thread may be in between)
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kSmemStatic);
+  if (e != cudaSuccess) return e;
+  if (max_attempts == 0) {
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, r.res.threads, r.res.smem);
+    return e != cudaSuccess ? e : per_sm > 0 ? cudaSuccess : cudaErrorCooperativeLaunchTooLarge;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)r.res.G);
+  cfg.blockDim = dim3((unsigned)r.res.threads);
+  cfg.dynamicSmemBytes = (size_t)r.res.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = r.res.G > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, d, r.res, max_attempts);
 }
 
 template <typename T, typename V, bool IMPLICIT>

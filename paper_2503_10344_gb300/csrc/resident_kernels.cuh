@@ -1,0 +1,601 @@
+// Step attempts of one LP held in the shared memory of all SMs (rows A4-A7 of the hot path;
+// float32 iterates, LPs of up to ~30 MB).
+//
+// An LP such as the 50,000 x 200,000 covering LP has 22 MB of step data: it sits in L2, and an
+// attempt of three dependent launches spends its 20 us on launch boundaries and on chains of
+// dependent loads (row pointer, column index, gathered entry), not on bytes.  Here one
+// cooperative launch runs a whole check period.  Block b of G owns a run of columns (rows of
+// A^T) and a run of rows of A, cut so that every block has about the same work (k_res_plan).
+// It copies their indices, values and vectors to shared memory once per launch; an attempt
+// then reads nothing from global memory but the gathered entries of y and of the (x', dx)
+// pairs:
+//   primal: the entries of y that the block's columns need, staged in shared memory, all loads
+//           in flight at once; then each column is summed in storage order (LANES lanes per
+//           row, rows beyond kResLong entries by a warp) and finished, its (x', dx) published;
+//   dual:   the same over the block's rows, y' published;
+//   the step decision (A6) by one thread of every block, from the same sums in the same order,
+//   so that all blocks hold bit-identical copies of the step state.
+// There is no grid barrier.  A published entry carries the number of the attempt that made it
+// (y and its tag in 8 bytes, x', dx and theirs in 16: single accesses), a gather reads an entry
+// again until the tag is the one it needs, and the blocks' partial sums travel the same way, one
+// 16-byte word per block.  So a phase starts on each entry as it arrives, without the four trips
+// to L2 that a fence, an arrival, a poll and a fence take (measured: 4,000-5,000 cycles per
+// barrier, two of them half of an attempt of the 2,000-row covering LP).  While one warp
+// collects the sums and decides, the others already gather the y' of this attempt: the next
+// primal step needs them if the step is accepted (a rejected step gathers the old y again).
+// No entry is overwritten while a block may still need it: x'(k + 1) is published after the
+// decision of attempt k, which has every block's sums, posted when its gathers of x'(k) were
+// done; y alternates between two buffers.
+// Every wait is bounded as in the cooperative kernel of iter_kernels.cuh.
+//
+// Measured per attempt on a GB300 (three launches -> here): see the table at auto_form() in
+// solver.cu, which chooses the form.
+#pragma once
+
+#include "internal.h"
+#include "iter_kernels.cuh"
+
+namespace pdlp {
+
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ ulonglong2 ld_relaxed_u128(const ulonglong2* p) {
+  ulonglong2 v;
+  asm volatile(
+      "{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+      : "=l"(v.x), "=l"(v.y)
+      : "l"(p)
+      : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_u128(ulonglong2* p, ulonglong2 v) {
+  asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
+               "l"(v.x), "l"(v.y)
+               : "memory");
+}
+__device__ __forceinline__ unsigned long long pack2(unsigned hi, float lo) {
+  return ((unsigned long long)hi << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ float low_f(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ unsigned high_u(unsigned long long v) { return (unsigned)(v >> 32); }
+
+// What a gather reads: a published y (tag | y) or pair (dx | x', tag in the second word).
+struct ResY {
+  using Word = unsigned long long;
+  using Acc = float;
+  static constexpr int kInFlight = kResGatherY;
+  static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u64(p); }
+  static __device__ __forceinline__ unsigned tag(const Word& w) { return high_u(w); }
+  static __device__ __forceinline__ Acc value(const Word& w) { return low_f(w); }
+};
+struct ResX {
+  using Word = ulonglong2;
+  using Acc = P2<float>;
+  static constexpr int kInFlight = kResGatherX;
+  static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u128(p); }
+  static __device__ __forceinline__ unsigned tag(const Word& w) { return (unsigned)w.y; }
+  static __device__ __forceinline__ Acc value(const Word& w) {
+    return Acc{low_f(w.x), __uint_as_float(high_u(w.x))};
+  }
+};
+
+// a bounded wait: false once the limit has passed or another block has given up
+struct ResWait {
+  DevState* st;
+  int limit, polls;
+  __device__ __forceinline__ bool more() {
+    if (++polls > limit) {
+      atomicExch(&st->bar_err, 1);
+      return false;
+    }
+    return (polls & 255) != 0 || *(volatile int*)&st->bar_err == 0;
+  }
+};
+
+// n / d for d > 0: the hardware's approximate reciprocal and one residual correction of the
+// quotient (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990): within an ulp in four instructions.
+__device__ __forceinline__ float div_pos(float n, float d) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+  const float q = n * r;
+  return fmaf(fmaf(-q, d, n), r, q);
+}
+
+// This block's three sums (lane-uniform) posted to every replica under `tag`, and the sums over
+// all blocks in slot order per lane, then a fixed shuffle tree.  Called by one whole warp.
+// (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.)
+__device__ __forceinline__ bool res_sums(DevState* st, ulonglong2* slot, int G, unsigned tag,
+                                         int limit, float (&sum)[3]) {
+  const int lane = threadIdx.x & 31, b = blockIdx.x;
+  if (lane < kResReplicas) {
+    const ulonglong2 w{pack2(tag, sum[0]), pack2(__float_as_uint(sum[2]), sum[1])};
+    st_relaxed_u128(slot + (size_t)lane * G + b, w);
+  }
+  const ulonglong2* mine = slot + (size_t)(b % kResReplicas) * G;
+  bool ok = true;
+  sum[0] = sum[1] = sum[2] = 0.f;
+  ResWait wait{st, limit, 0};
+  for (int b0 = 0; b0 < G; b0 += 32 * kResPoll) {
+    ulonglong2 w[kResPoll];
+#pragma unroll
+    for (int i = 0; i < kResPoll; ++i)
+      if (b0 + i * 32 + lane < G) w[i] = ld_relaxed_u128(mine + b0 + i * 32 + lane);
+    bool miss = true;
+    while (miss) {
+      miss = false;
+#pragma unroll
+      for (int i = 0; i < kResPoll; ++i)
+        if (b0 + i * 32 + lane < G && high_u(w[i].x) != tag) {
+          miss = true;
+          w[i] = ld_relaxed_u128(mine + b0 + i * 32 + lane);
+        }
+      if (miss && !wait.more()) {
+        ok = false;
+        break;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kResPoll; ++i)
+      if (b0 + i * 32 + lane < G) {
+        sum[0] += low_f(w[i].x);
+        sum[1] += low_f(w[i].y);
+        sum[2] += __uint_as_float(high_u(w[i].y));
+      }
+  }
+  ok = __all_sync(0xffffffffu, ok);
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+  return ok;
+}
+
+// One side's rows of the block.
+template <typename V>
+struct ResSide {
+  const int* ptr;       // [rows + 1] relative to the block's first nonzero
+  const unsigned* key;  // [nnz] the gathers: index | (place in the chunk << bits)
+  const V* val;         // [nnz] values in storage order (none for a pattern)
+  const int* lng;       // [nlong] rows longer than kResLong
+  int rows, nlong, bits, cap;
+};
+
+template <typename V>
+__device__ __forceinline__ float res_val(const V* v, int p) {
+  if constexpr (std::is_same<V, Pattern>::value) return 1.f;
+  else if constexpr (std::is_same<V, float>::value) return v[p];
+  else return __bfloat162float(v[p]);
+}
+
+// The chunk of whole rows from row ra: at most `cap` nonzeros (every thread finds its end).
+__device__ __forceinline__ int res_chunk_end(const int* ptr, int rows, int cap, int ra) {
+  const int p0 = ptr[ra];
+  if (ptr[rows] - p0 <= cap) return rows;
+  int lo = ra + 1, hi = rows;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (ptr[mid] - p0 <= cap) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// The gathers of a chunk in the order of the entries they read, to 2^shift entries: a warp's
+// loads then share cache lines (unordered, each lane's load is a line of its own and the SM
+// looks up one a cycle: 8,900 gathers of the covering LP's y per SM took 12,300 cycles).
+// hist[kResBuckets]: scratch.  The order within a bucket is whatever the counters give: it does
+// not enter any result.
+__device__ __forceinline__ void res_sort_keys(const int* __restrict__ col, int n, int shift,
+                                              int bits, int* hist, unsigned* key) {
+  __shared__ int wsum[32];
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+  for (int i = tid; i < kResBuckets; i += T) hist[i] = 0;
+  __syncthreads();
+  for (int p = tid; p < n; p += T) atomicAdd(hist + (__ldg(col + p) >> shift), 1);
+  __syncthreads();
+  // exclusive scan: each thread a run of kResBuckets / T buckets
+  const int per = kResBuckets / T;
+  int s = 0;
+  for (int k = 0; k < per; ++k) s += hist[tid * per + k];
+  int inc = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) wsum[tid >> 5] = inc;
+  __syncthreads();
+  int base = inc - s;
+  for (int w = 0; w < (tid >> 5); ++w) base += wsum[w];
+  for (int k = 0; k < per; ++k) {
+    const int c = hist[tid * per + k];
+    hist[tid * per + k] = base;
+    base += c;
+  }
+  __syncthreads();
+  for (int p = tid; p < n; p += T) {
+    const int c = __ldg(col + p);
+    key[atomicAdd(hist + (c >> shift), 1)] = (unsigned)c | ((unsigned)p << bits);
+  }
+  __syncthreads();
+}
+
+// Sums over the staged entries of rows [ra, rb) of the chunk that starts at nonzero p0, and
+// their epilogues: LANES lanes per row, then a warp per long row.
+template <int LANES, typename Acc, typename V, typename Fin>
+__device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, int p0, int ra,
+                                         int rb, Fin fin) {
+  const int lane = threadIdx.x & (LANES - 1), T = blockDim.x;
+  auto add = [&](Acc& acc, int p) {
+    const float v = res_val<V>(s.val, p);
+    const Acc t = stage[p - p0];
+    if constexpr (std::is_same<Acc, float>::value) acc += v * t;
+    else acc += Acc{v * t.a, v * t.b};
+  };
+  for (int r = ra + (int)threadIdx.x / LANES; r < rb; r += T / LANES) {
+    const int b = s.ptr[r], e = s.ptr[r + 1];
+    if (e - b > kResLong) continue;  // uniform within the group
+    Acc acc{};
+#pragma unroll 4
+    for (int p = b + lane; p < e; p += LANES) add(acc, p);
+    acc = group_sum<LANES>(acc);
+    if (lane == 0) fin(r, acc);
+  }
+  const int wl = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < s.nlong; k += T >> 5) {
+    const int r = s.lng[k];
+    if (r < ra || r >= rb) continue;
+    const int b = s.ptr[r], e = s.ptr[r + 1];
+    Acc acc{};
+#pragma unroll 4
+    for (int p = b + wl; p < e; p += 32) add(acc, p);
+    acc = group_sum<32>(acc);
+    if (wl == 0) fin(r, acc);
+  }
+}
+
+template <typename Acc, typename V, typename Fin>
+__device__ __forceinline__ void res_rows_lanes(int lanes, const ResSide<V>& s, const Acc* stage,
+                                               int p0, int ra, int rb, Fin fin) {
+  switch (lanes) {
+    case 1: return res_rows<1>(s, stage, p0, ra, rb, fin);
+    case 2: return res_rows<2>(s, stage, p0, ra, rb, fin);
+    case 4: return res_rows<4>(s, stage, p0, ra, rb, fin);
+    case 8: return res_rows<8>(s, stage, p0, ra, rb, fin);
+    default: return res_rows<16>(s, stage, p0, ra, rb, fin);
+  }
+}
+
+// The entries that the rows of a chunk need, into the stage: threads t, t + nt, ... of the
+// block, E::kInFlight loads in flight each.  Returns false when a wait gave up.
+// (A newer tag ends the wait too: only the y gathered ahead of a step that is then rejected can
+// meet one, and it is dropped.)
+template <typename E, typename V>
+__device__ __forceinline__ bool res_gather(const ResSide<V>& s, int p0, int n,
+                                           const typename E::Word* __restrict__ from, unsigned tag,
+                                           typename E::Acc* stage, int t, int nt, ResWait wait) {
+  constexpr int U = E::kInFlight;
+  const unsigned mask = (1u << s.bits) - 1u;
+  const unsigned* key = s.key + p0;
+  for (int i0 = t; i0 < n; i0 += nt * U) {
+    unsigned c[U];
+    typename E::Word w[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) c[k] = i0 + k * nt < n ? key[i0 + k * nt] : 0u;
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (i0 + k * nt < n) w[k] = E::load(from + (c[k] & mask));
+    bool miss = true;
+    while (miss) {
+      miss = false;
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (i0 + k * nt < n && (int)(E::tag(w[k]) - tag) < 0) {
+          miss = true;
+          w[k] = E::load(from + (c[k] & mask));
+        }
+      if (miss && !wait.more()) return false;
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (i0 + k * nt < n) stage[c[k] >> s.bits] = E::value(w[k]);
+  }
+  return true;
+}
+
+// A side's product: chunk by chunk the entries its rows need, then the rows' sums.  The first
+// chunk may have been gathered ahead (`ahead`).
+template <typename E, typename V, typename Fin>
+__device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
+                                            const typename E::Word* from, unsigned tag,
+                                            typename E::Acc* stage, bool ahead, ResWait wait,
+                                            int* fail, Fin fin) {
+  int ra = 0;
+  while (ra < s.rows) {
+    const int p0 = s.ptr[ra], rb = res_chunk_end(s.ptr, s.rows, s.cap, ra);
+    if (ra > 0) __syncthreads();  // the chunk before is summed
+    if (ra > 0 || !ahead)
+      if (!res_gather<E>(s, p0, s.ptr[rb] - p0, from, tag, stage, threadIdx.x, blockDim.x, wait))
+        *fail = 1;
+    __syncthreads();
+    res_rows_lanes<typename E::Acc>(lanes, s, stage, p0, ra, rb, fin);
+    ra = rb;
+  }
+}
+
+// The step decision (decide_step in float32, the same operations) in two halves: what the next
+// attempt reads, which every thread of the block waits for, and the rest of the state, which
+// the deciding thread writes while the others go on.
+struct ResDecision {
+  float eta, eta_bar, eta_next;
+  bool accept;
+};
+__device__ __forceinline__ ResDecision res_decide(DevState* st, float dx2, float dy2, float dkd,
+                                                  float fd, float fi, int& left) {
+  ResDecision r{st->eta_f, INFINITY, st->eta_f, true};
+  if (!isfinite(dx2) || !isfinite(dy2) || !isfinite(dkd)) {
+    st->status = 4;  // PDLP_NUMERICAL
+    return r;
+  }
+  const float om = st->omega_f, iom = st->inv_omega_f;
+  if (st->adaptive || st->tr_cap > 0) {  // (a fixed step needs the bound for the trace alone)
+    const float den = 2.f * fabsf(dkd);
+    r.eta_bar = den > 0.f ? (om * dx2 + dy2 * iom) / den : INFINITY;
+  }
+  if (st->adaptive) {
+    r.eta_next = fminf(fd * r.eta_bar, fi * r.eta);
+    r.accept = !(r.eta > r.eta_bar);
+  }
+  if (r.accept) {
+    st->cur ^= 1;
+    st->pw_f = r.eta;
+    if (--left == 0) st->check_due = 1;
+  } else {
+    st->pw_f = 0.f;
+  }
+  st->eta_f = r.eta_next;
+  st->tau_f = r.eta_next * iom;
+  st->sigma_f = r.eta_next * om;
+  return r;
+}
+__device__ __forceinline__ void res_record(DevState* st, const ResDecision& r) {
+  const long long t = st->attempts;
+  st->attempts = t + 1;
+  if (st->status == 4) return;
+  if (t < st->tr_cap) {
+    st->tr_eta[t] = (double)r.eta;
+    st->tr_eta_bar[t] = (double)r.eta_bar;
+    st->tr_accepted[t] = r.accept ? 1 : 0;
+  }
+  if (r.accept) {
+    st->pending_w = (double)r.eta;
+    st->sum_w += (double)r.eta;
+    st->iters += 1;
+  } else {
+    st->pending_w = 0.0;
+  }
+  st->eta = (double)r.eta_next;
+}
+
+template <typename V, bool IMPLICIT>
+__global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d, ResPlan R,
+                                                           int max_attempts) {
+  constexpr bool VALS = !std::is_same<V, Pattern>::value;
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ DevState ls;
+  __shared__ float red[3][32];  // the warps' sums (0 beyond the block's warps)
+  __shared__ int nlong[2], stop, fail;
+  DevState* gst = d.st;
+  const int tid = threadIdx.x, T = blockDim.x, G = R.G, b = blockIdx.x;
+  if (tid == 0) {
+    ls = *gst;
+    if (b != 0) ls.tr_cap = 0;  // one block writes the trace
+    stop = (ls.status != 0 || ls.check_due) ? 1 : 0;
+    fail = 0;
+  }
+  if (tid < 32) red[0][tid] = red[1][tid] = red[2][tid] = 0.f;
+  __syncthreads();
+  if (stop) return;
+  // ---- the block's columns [t0, t1) and rows [a0, a1)
+  const int t0 = R.cut_t[b], t1 = R.cut_t[b + 1], a0 = R.cut_a[b], a1 = R.cut_a[b + 1];
+  const int nt = t1 - t0, na = a1 - a0;
+  const int tz0 = __ldg(d.t_ptr + t0), az0 = __ldg(d.a_ptr + a0);
+  const int tz = __ldg(d.t_ptr + t1) - tz0, az = __ldg(d.a_ptr + a1) - az0;
+  const ResLayout L = res_layout(nt, tz, na, az, VALS ? (int)sizeof(V) : 0, IMPLICIT);
+  int* tp = (int*)(sm + L.t_ptr);
+  unsigned* tk = (unsigned*)(sm + L.t_col);
+  V* tv = VALS ? (V*)(sm + L.t_val) : nullptr;
+  int* tl = (int*)(sm + L.t_lng);
+  int* ap = (int*)(sm + L.a_ptr);
+  unsigned* ak = (unsigned*)(sm + L.a_col);
+  V* av = VALS ? (V*)(sm + L.a_val) : nullptr;
+  int* al = (int*)(sm + L.a_lng);
+  float* c = (float*)(sm + L.c);
+  float* l = (float*)(sm + L.l);
+  float* u = (float*)(sm + L.u);
+  float* tw = IMPLICIT ? (float*)(sm + L.tw) : nullptr;
+  float* q = (float*)(sm + L.q);
+  float* sw = IMPLICIT ? (float*)(sm + L.sw) : nullptr;
+  unsigned char* kind = sm + L.kind;
+  float* xs[2] = {(float*)(sm + L.x0), (float*)(sm + L.x1)};
+  float* ys[2] = {(float*)(sm + L.y0), (float*)(sm + L.y1)};
+  float* sx = (float*)(sm + L.sx);
+  float* sy = (float*)(sm + L.sy);
+  P2<float>* stage2 = (P2<float>*)(sm + L.bytes);
+  float* stage1 = (float*)(sm + L.bytes);
+  // ---- copy in (iterates with ordinary loads: the KKT block of the same graph wrote them);
+  // the y of this launch is published under a tag of its own
+  for (int i = tid; i <= nt; i += T) tp[i] = __ldg(d.t_ptr + t0 + i) - tz0;
+  for (int i = tid; i <= na; i += T) ap[i] = __ldg(d.a_ptr + a0 + i) - az0;
+  const int cur0 = ls.cur;
+  const unsigned tag0 = 2u * (unsigned)ls.attempts;
+  for (int i = tid; i < na; i += T) {
+    const float y = d.y[cur0][a0 + i];
+    st_relaxed_u64(R.ex_y[cur0] + a0 + i, pack2(tag0 + 1u, y));
+    ys[cur0][i] = y;
+    q[i] = __ldg(d.q + a0 + i);
+    if constexpr (IMPLICIT) sw[i] = __ldg(d.sw + a0 + i);
+    kind[i] = __ldg(d.row_kind + a0 + i);
+    sy[i] = d.sum_y[a0 + i];
+  }
+  for (int j = tid; j < nt; j += T) {
+    c[j] = __ldg(d.c + t0 + j);
+    l[j] = __ldg(d.l + t0 + j);
+    u[j] = __ldg(d.u + t0 + j);
+    if constexpr (IMPLICIT) tw[j] = __ldg(d.tw + t0 + j);
+    xs[cur0][j] = d.x[cur0][t0 + j].x;
+    sx[j] = d.sum_x[t0 + j];
+  }
+  if constexpr (VALS) {
+    for (int p = tid; p < tz; p += T) tv[p] = d.t_val[tz0 + p];
+    for (int p = tid; p < az; p += T) av[p] = d.a_val[az0 + p];
+  }
+  __syncthreads();
+  // the gathers of every chunk, ordered
+  int* hist = (int*)stage1;
+  for (int ra = 0; ra < nt;) {
+    const int rb = res_chunk_end(tp, nt, R.cap_t, ra), p0 = tp[ra];
+    res_sort_keys(d.t_col + tz0 + p0, tp[rb] - p0, R.shift_t, R.bits_t, hist, tk + p0);
+    ra = rb;
+  }
+  for (int ra = 0; ra < na;) {
+    const int rb = res_chunk_end(ap, na, R.cap_a, ra), p0 = ap[ra];
+    res_sort_keys(d.a_col + az0 + p0, ap[rb] - p0, R.shift_a, R.bits_a, hist, ak + p0);
+    ra = rb;
+  }
+  // the long rows of each side in order (one warp per side)
+  if (tid < 64) {
+    const int side = tid >> 5, lane = tid & 31, n = side ? na : nt;
+    const int* ptr = side ? ap : tp;
+    int* lst = side ? al : tl;
+    int cnt = 0;
+    for (int r0 = 0; r0 < n; r0 += 32) {
+      const int r = r0 + lane;
+      const bool lg = r < n && ptr[r + 1] - ptr[r] > kResLong;
+      const unsigned m = __ballot_sync(0xffffffffu, lg);
+      if (lg) lst[cnt + __popc(m & ((1u << lane) - 1u))] = r;
+      cnt += __popc(m);
+    }
+    if (lane == 0) nlong[side] = cnt;
+  }
+  // accepted steps to the next check (thread 0)
+  int left = 0;
+  if (tid == 0) {
+    const long long p = ls.period - ls.iters % ls.period, q = ls.iter_limit - ls.iters;
+    left = (int)(p < q ? p : q > 1 ? q : 1);
+  }
+  __syncthreads();
+  const ResSide<V> st{tp, tk, tv, tl, nt, nlong[0], R.bits_t, R.cap_t};
+  const ResSide<V> sa{ap, ak, av, al, na, nlong[1], R.bits_a, R.cap_a};
+  const int ahead_n = nt ? tp[res_chunk_end(tp, nt, R.cap_t, 0)] : 0;  // the first chunk of st
+  const ResWait wait{gst, (int)ls.spin_limit, 0};
+  ResDecision dec{};
+  unsigned ytag = tag0 + 1u;
+  bool ahead = false;  // the first chunk of the next primal step is staged
+  for (int att = 0; att < max_attempts; ++att) {
+    const int cur = ls.cur;
+    const float pw = ls.pw_f, tau = ls.tau_f, sigma = ls.sigma_f;
+    const unsigned tag = tag0 + 2u * (unsigned)(att + 1);
+    float fd = 0.f, fi = 0.f;
+    if (tid == 0) {
+      if (att > 0) res_record(&ls, dec);  // of the attempt before
+      step_factors(&ls, ls.attempts + 1, &fd, &fi);
+    }
+    // ---- A4: primal step over the block's columns
+    {
+      const float* xo = xs[cur];
+      float* xn = xs[cur ^ 1];
+      float dx2 = 0.f;
+      auto fin = [&](int j, float aty) {
+        const float x = xo[j];
+        const float w = IMPLICIT ? tw[j] : 1.f;
+        const float step = IMPLICIT ? tau * w : tau;
+        const float xv = clampv(x - step * (c[j] - aty), l[j], u[j]);
+        const float dd = xv - x;
+        xn[j] = xv;
+        st_relaxed_u128(R.ex_x + t0 + j, ulonglong2{pack2(__float_as_uint(dd), xv), tag});
+        if (pw != 0.f) sx[j] += pw * x;  // A7: add the iterate whose weight is pending
+        dx2 += IMPLICIT ? div_pos(dd * dd, w) : dd * dd;
+      };
+      res_product<ResY>(R.lanes_t, st, R.ex_y[cur], ytag, stage1, ahead, wait, &fail, fin);
+      dx2 = group_sum<32>(dx2);
+      if ((tid & 31) == 0) red[0][tid >> 5] = dx2;
+    }
+    __syncthreads();  // the stage is free
+    // ---- A5: dual step over the block's rows
+    {
+      const float* yo = ys[cur];
+      float* yn = ys[cur ^ 1];
+      unsigned long long* gy = R.ex_y[cur ^ 1];
+      float dy2 = 0.f, dkd = 0.f;
+      auto fin = [&](int i, P2<float> acc) {  // acc.a = (K x')_i, acc.b = (K dx)_i
+        const float y = yo[i];
+        const float w = IMPLICIT ? sw[i] : 1.f;
+        const float step = IMPLICIT ? sigma * w : sigma;
+        float yv = y + step * (q[i] - (acc.a + acc.b));
+        if (kind[i] != 1) yv = fmaxf(yv, 0.f);
+        st_relaxed_u64(gy + a0 + i, pack2(tag, yv));
+        yn[i] = yv;
+        if (pw != 0.f) sy[i] += pw * y;
+        const float dd = yv - y;
+        dy2 += IMPLICIT ? div_pos(dd * dd, w) : dd * dd;
+        dkd += dd * acc.b;
+      };
+      res_product<ResX>(R.lanes_a, sa, R.ex_x, tag, stage2, false, wait, &fail, fin);
+      dy2 = group_sum<32>(dy2);
+      dkd = group_sum<32>(dkd);
+      if ((tid & 31) == 0) {
+        red[1][tid >> 5] = dy2;
+        red[2][tid >> 5] = dkd;
+      }
+    }
+    __syncthreads();  // the stage is free, the warps' sums are there
+    if (tid < 32) {
+      float s[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s[k] = group_sum<32>(red[k][tid]);
+      bool ok = fail == 0;
+      if (G > 1) ok = res_sums(gst, R.slot, G, tag, wait.limit, s) && ok;
+      // ---- A6: the same decision in every block
+      if (tid == 0) {
+        dec = res_decide(&ls, s[0], s[1], s[2], fd, fi, left);
+        stop = !ok ? 2 : (ls.status != 0 || ls.check_due) ? 1 : 0;
+      }
+    } else if (!res_gather<ResY>(st, 0, ahead_n, R.ex_y[cur ^ 1], tag, stage1, tid - 32, T - 32,
+                                 wait)) {
+      fail = 1;
+    }
+    __syncthreads();
+    if (stop || fail) break;
+    ahead = ls.cur != cur;  // accepted: what was gathered ahead is the y of the next step
+    if (ahead) ytag = tag;
+    if (!ahead) __syncthreads();  // the stage is gathered anew
+  }
+  if (stop == 2 || fail) {  // a wait gave up: so do the others', before long
+    if (tid == 0) {
+      atomicExch(&gst->bar_err, 1);
+      atomicExch(&gst->status, kStatusWaitFailed);
+    }
+    return;
+  }
+  if (tid == 0 && max_attempts > 0) res_record(&ls, dec);  // of the last attempt
+  // ---- copy out: the iterate (its step is not needed any more) and the running sums
+  const int cur = ls.cur;
+  for (int j = tid; j < nt; j += T) {
+    d.x[cur][t0 + j] = make_float2(xs[cur][j], 0.f);
+    d.sum_x[t0 + j] = sx[j];
+  }
+  for (int i = tid; i < na; i += T) {
+    d.y[cur][a0 + i] = ys[cur][i];
+    d.sum_y[a0 + i] = sy[i];
+  }
+  if (b == 0 && tid == 0) store_step_state(gst, ls);
+}
+
+}  // namespace pdlp

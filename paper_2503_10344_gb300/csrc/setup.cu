@@ -1207,6 +1207,60 @@ cudaError_t setup_len_order(const int* ptr, int rows, int* ord, cudaStream_t s) 
   return cudaGetLastError();
 }
 
+// Cuts of the resident step kernel: block g's rows start where the nonzeros and kResRowWeight
+// per row before them reach g / G of the total, so that the blocks' gathers and epilogues are
+// even (an epilogue costs about as much as four gathered entries).  Block 0 finds the cuts, every
+// block looks for the longest row.
+constexpr int kResRowWeight = 4;
+__global__ void __launch_bounds__(kBlock) k_res_plan(int m, int n, long long nnz,
+                                                     const int* a_ptr, const int* t_ptr, int G,
+                                                     int vb, int implicit, int* cut_t, int* cut_a,
+                                                     ResSizes* sizes) {
+  int longest = 0;
+  const long long stride = (long long)gridDim.x * kBlock;
+  for (long long i = (long long)blockIdx.x * kBlock + threadIdx.x; i < (long long)m + n;
+       i += stride) {
+    const int* p = i < m ? a_ptr + i : t_ptr + (i - m);
+    longest = max(longest, p[1] - p[0]);
+  }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if ((threadIdx.x & 31) == 0) atomicMax(&sizes->max_len, longest);
+  if (blockIdx.x != 0) return;
+  const int g = threadIdx.x;
+  for (int side = 0; side < 2; ++side) {
+    const int rows = side ? m : n;
+    const int* ptr = side ? a_ptr : t_ptr;
+    int* cut = side ? cut_a : cut_t;
+    if (g <= G) {
+      const long long want = (nnz + (long long)kResRowWeight * rows) * g / G;
+      int lo = 0, hi = rows;  // the first row whose weight before it is at least `want`
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (ptr[mid] + (long long)kResRowWeight * mid >= want) hi = mid; else lo = mid + 1;
+      }
+      cut[g] = lo;
+    }
+  }
+  __syncthreads();
+  if (g < G) {
+    const int nt = cut_t[g + 1] - cut_t[g], zt = t_ptr[cut_t[g + 1]] - t_ptr[cut_t[g]];
+    const int na = cut_a[g + 1] - cut_a[g], za = a_ptr[cut_a[g + 1]] - a_ptr[cut_a[g]];
+    atomicMax(&sizes->t_rows, nt);
+    atomicMax(&sizes->t_nnz, zt);
+    atomicMax(&sizes->a_rows, na);
+    atomicMax(&sizes->a_nnz, za);
+    atomicMax(&sizes->bytes, res_layout(nt, zt, na, za, vb, implicit != 0).bytes);
+  }
+}
+
+cudaError_t setup_res_plan(int m, int n, int nnz, const int* a_ptr, const int* t_ptr, int G, int vb,
+                           bool implicit, int* cut_t, int* cut_a, ResSizes* sizes, cudaStream_t s) {
+  RET(cudaMemsetAsync(sizes, 0, sizeof(ResSizes), s));
+  k_res_plan<<<grid_for((long long)m + n, device_sm_count()), kBlock, 0, s>>>(
+      m, n, nnz, a_ptr, t_ptr, G, vb, implicit ? 1 : 0, cut_t, cut_a, sizes);
+  return cudaGetLastError();
+}
+
 cudaError_t setup_rescale(int m, int n, int fp32, double beta, double gamma, void* c, void* l,
                           void* u, void* q, void* x0, void* y0, double* dr, double* dc,
                           double* inv_dr, double* inv_dc, cudaStream_t s) {

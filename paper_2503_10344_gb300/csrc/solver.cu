@@ -103,6 +103,7 @@ struct Bufs {
   double2 *ndg_gx, *ndg_gy;  // normalized-duality-gap restarts (NULL off)
   NdgState* ndg;
   double* ndg_part;
+  size_t tmp_bytes;  // of tmp
 };
 
 constexpr int kMaxLongBlocks = 1024;
@@ -198,7 +199,8 @@ static size_t carve(Arena& ar, Bufs& b, int m, int n, long long nnz, int precisi
     b.tlp_t = (int*)ar.take(4 * 4);
     tile_tmp = tile_tmp_ints(std::max(m, n));
   }
-  b.tmp = (int*)ar.take(4 * std::max(tmp_ints, tile_tmp));
+  b.tmp_bytes = 4 * std::max(tmp_ints, tile_tmp);
+  b.tmp = (int*)ar.take(b.tmp_bytes);
   // normalized-duality-gap restarts: gradients of both candidates, bisection state, partials
   b.ndg_gx = ndg ? (double2*)ar.take(16 * N) : nullptr;
   b.ndg_gy = ndg ? (double2*)ar.take(16 * M) : nullptr;
@@ -291,6 +293,13 @@ struct Solve {
   cudaError_t persist(int max_attempts) {
     ++g_launches;
     int g = 0;
+    if (ir.res.G > 0) {
+      switch (mode) {
+        case MODE_FP32: return launch_resident_fp32(ir, max_attempts, s);
+        case MODE_BF16: return launch_resident_bf16(ir, max_attempts, s);
+        default: return launch_resident_pat(ir, max_attempts, s);
+      }
+    }
     switch (mode) {
       case MODE_FP64: return launch_persist_fp64(lanes_a, lanes_t, ir, max_attempts, persist_grid, &g, s);
       case MODE_FP32: return launch_persist_fp32(lanes_a, lanes_t, ir, max_attempts, persist_grid, &g, s);
@@ -457,7 +466,60 @@ struct SetupOut {
                   // columns with an infinite bound
   int lanes_a, lanes_t, lanes_ka, lanes_kt, th_a, th_t, nlong_a, nlong_t;
   int tiles, n_ta, n_tt;  // staged tile kernels built; their items over A and A^T
+  int res_G;              // blocks of the resident step kernel (0: not planned)
+  void* res_base;         // its buffers
+  ResSizes res;
 };
+
+// The form of the step attempts of one LP with float32 iterates where the caller asks for none
+// (persistent = 0 without lanes, tiles, the autotuner or the Halpern variant): the LP in one
+// block's shared memory up to kOneBlockNnz nonzeros, spread over the SMs' shared memory
+// (resident_kernels.cuh) while it fits there, else three launches per attempt.  Measured per
+// attempt on a GB300 (us; values in float32 / bfloat16 or the 0/1 pattern):
+//                                 nonzeros   three launches   one block     resident
+//   relaxation 200 x 400             1,670      9.9 /  9.4    2.5 /  2.8    3.8 /  3.7
+//   relaxation 400 x 800             3,238     10.0 /  9.6    3.9 /  4.6    3.7 /  3.7
+//   relaxation 2,000 x 4,000        15,963     13.4 / 12.0   30.3 / 36.4    4.4 /  4.5
+//   covering 2,000 x 8,000          54,130     12.4 / 11.6                  5.0 /  5.0
+//   covering 10,000 x 40,000       269,989     14.2 / 13.0                  6.6 /  6.4
+//   covering 50,000 x 200,000    1,350,409     23.0 / 20.5                 20.3 / 13.7
+//   energy system, 24 h             21,600     23.3                         4.9
+//   energy system, 720 h           648,000     17.7                        10.4
+// kResNnz nonzeros per block: 256 and 1,024 measured within 10 % of 512, slower on most.
+constexpr int kResNnz = 512;
+constexpr int kOneBlockNnz = 2500;
+static bool auto_form(const pdlp_params* p, Mode mode, int m, long long nnz) {
+  return mode != MODE_FP64 && p->persistent == 0 && !p->tiles && !p->halpern && !p->autotune &&
+         !p->lanes_A && !p->lanes_AT && m > 0 && nnz > 0;
+}
+static int resident_blocks(long long nnz) {
+  return (int)std::max(1LL, std::min<long long>(device_sm_count(), nnz / kResNnz));
+}
+// Buffers of the resident step kernel, from `base` on (256-byte aligned).
+struct ResBufs {
+  ulonglong2 *slot, *ex_x;
+  unsigned long long* ex_y;  // [2][m]
+  int *cut_t, *cut_a;
+  ResSizes* sizes;
+  size_t clear, bytes;  // the first `clear` bytes start as zeros (no tag)
+  ResBufs(void* base, int G, long long m, long long n) {
+    Arena ar{(char*)base, 0};
+    slot = (ulonglong2*)ar.take(16 * (size_t)kResReplicas * G);
+    ex_x = (ulonglong2*)ar.take(16 * (size_t)n);
+    ex_y = (unsigned long long*)ar.take(8 * 2 * (size_t)m);
+    clear = ar.off;
+    cut_t = (int*)ar.take(4 * ((size_t)G + 1));
+    cut_a = (int*)ar.take(4 * ((size_t)G + 1));
+    sizes = (ResSizes*)ar.take(sizeof(ResSizes));
+    bytes = ar.off;
+  }
+};
+static int optin_smem() {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return optin;
+}
 
 // Validation, canonical form, transpose, value format, scaling, iteration-space
 // data and long-row lists of one LP.  forced_mode >= 0 skips the value-format
@@ -564,6 +626,28 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
     if (m > 0) CUDA_TRY(setup_long_rows(bf.a_ptr, m, th_a, flags, pos, bsum, bf.a_long, &nlong_a, s));
     CUDA_TRY(setup_long_rows(bf.t_ptr, n, th_t, flags, pos, bsum, bf.t_long, &nlong_t, s));
     g_launches += 10;
+  }
+  // the parts of the resident step kernel, if the LP's data can fit on the chip at all and its
+  // buffers in scratch that is free by now: the scalars' partial sums or the transpose's
+  so->res_G = 0;
+  so->res_base = nullptr;
+  so->res = ResSizes{};
+  if (auto_form(p, mode, m, nnz) && nnz > kOneBlockNnz) {
+    const int vb = mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
+    const long long data = nnz * 2 * (4 + vb) + 24LL * ((long long)m + n);
+    const int G = resident_blocks(nnz);
+    const size_t need = ResBufs(nullptr, G, m, n).bytes;
+    so->res_base = need <= 8 * setup_part_doubles(m, n) ? (void*)bf.part_setup
+                   : need <= bf.tmp_bytes               ? (void*)bf.tmp
+                                                        : nullptr;
+    if (so->res_base && data <= (long long)device_sm_count() * optin_smem()) {
+      so->res_G = G;
+      const ResBufs rb(so->res_base, G, m, n);
+      CUDA_TRY(setup_res_plan(m, n, (int)nnz, bf.a_ptr, bf.t_ptr, G, vb, mode != MODE_FP32,
+                              rb.cut_t, rb.cut_a, rb.sizes, s));
+      CUDA_TRY(cudaMemcpyAsync(&so->res, rb.sizes, sizeof(ResSizes), cudaMemcpyDeviceToHost, s));
+      ++g_launches;
+    }
   }
   // work items of the staged tile kernels (float32 iterates)
   so->tiles = 0;
@@ -1048,12 +1132,67 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
                                   set_dry);
     if (rc) return rc;
   }
-  if (p->persistent) {
+  if (so.res_G > 0) {
+    // an LP that fits in the SMs' shared memory
+    const ResBufs rb(so.res_base, so.res_G, m, n);
+    const ResSizes& z = so.res;
+    ResPlan R{};
+    R.G = so.res_G;
+    R.cut_t = rb.cut_t;
+    R.cut_a = rb.cut_a;
+    R.slot = rb.slot;
+    R.ex_x = rb.ex_x;
+    R.ex_y[0] = rb.ex_y;
+    R.ex_y[1] = rb.ex_y + m;
+    auto bits = [](long long count) {  // bits of an index below count
+      int k = 1;
+      while ((1LL << k) < count) ++k;
+      return k;
+    };
+    R.bits_t = bits(m);
+    R.bits_a = bits(n);
+    R.shift_t = std::max(0, R.bits_t - bits(kResBuckets));
+    R.shift_a = std::max(0, R.bits_a - bits(kResBuckets));
+    const int part = std::max(z.t_nnz, z.a_nnz);
+    R.threads = part <= 1024 ? 256 : kResBlock;
+    auto lanes = [&](int rows) {  // as many lanes per row as one round of the block allows
+      int L = 1;
+      while (L < 16 && 2LL * L * rows <= R.threads) L <<= 1;
+      return L;
+    };
+    R.lanes_t = lanes(z.t_rows);
+    R.lanes_a = lanes(z.a_rows);
+    // the stage: a side's whole part where it fits, else as much as does (whole rows)
+    const long long room = optin_smem() - kSmemStatic - (long long)z.bytes;
+    const long long want =
+        (std::max({4LL * z.t_nnz, 8LL * z.a_nnz, 4LL * kResBuckets}) + 15) / 16 * 16;
+    const long long stage = std::min(want, room / 16 * 16);
+    R.cap_t = (int)(stage / 4);
+    R.cap_a = (int)(stage / 8);
+    R.smem = (int)(z.bytes + stage);
+    const bool fits = stage == want || stage >= 8LL * std::max(z.max_len, kResMinStage);
+    if (fits && R.bits_t + bits(z.t_nnz) <= 32 && R.bits_a + bits(z.a_nnz) <= 32) {
+      sv.ir.res = R;
+      sv.persist_grid = R.G;
+      if (sv.persist(0) != cudaSuccess) {  // asks whether the blocks can be resident
+        sv.ir.res = ResPlan{};
+        sv.persist_grid = 0;
+      } else {
+        CUDA_TRY(cudaMemsetAsync(rb.slot, 0, rb.clear, s));
+      }
+    }
+  }
+  // one block: asked for, or a small LP whose form is ours to choose (and which fits: below)
+  const bool small = auto_form(p, mode, m, nnz) && nnz <= kOneBlockNnz &&
+                     smem_layout(m, n, nnz, 4, mode != MODE_PAT, mode != MODE_FP32).bytes <=
+                         optin_smem() - kSmemStatic;
+  if (p->persistent || small) {
     // the resident grid of the persistent kernel (probe launch with nothing to do:
     // the state says check_due, so every block returns at entry)
     // persistent = 2: one block (small LPs: the grid barrier is the block's barrier)
-    const int want = p->persistent == 2 ? 1 : 0;
-    if (p->persistent == 2) {
+    const bool one = p->persistent == 2 || small;
+    const int want = one ? 1 : 0;
+    if (one) {
       // the one block holds the LP in shared memory when it fits (the 200 x 400
       // relaxations take 76 KB in float64), else it steps from global memory
       int dev = 0, optin = 0;
@@ -1313,7 +1452,9 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
   r->lanes_A = sv.lanes_a;
   r->lanes_AT = sv.lanes_t;
   r->tiles = sv.ir.tile;
-  r->persistent_form = p->persistent == 0 ? 0 : p->persistent == 1 ? 1 : sv.ir.smem.bytes > 0 ? 3 : 2;
+  r->persistent_form = sv.ir.res.G > 0       ? 4
+                       : sv.ir.smem.bytes > 0 ? 3
+                       : p->persistent;
   r->spectral_norm = spectral;
   r->iters = fs.iters;
   r->attempts = fs.attempts;
@@ -1385,7 +1526,10 @@ static int time_kernels_after_setup(Solve& sv, DevState* st, int mode, long long
     cudaGraph_t g;
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     cudaError_t ce = cudaSuccess;
-    if (which == 5) ce = cap.persist(tq.reps);  // reps attempts inside one launch
+    // reps attempts inside one launch (posted words of an earlier run would carry its tags)
+    if (which == 5 && sv.ir.res.G > 0)
+      ce = cudaMemsetAsync(sv.ir.res.slot, 0, ResBufs(sv.ir.res.slot, sv.ir.res.G, m, n).clear, cs);
+    if (which == 5 && ce == cudaSuccess) ce = cap.persist(tq.reps);
     for (int i = 0; i < tq.reps && ce == cudaSuccess && which != 5; ++i) {
       if (which == 0 || which == 2) ce = cap.iter(IK_PRIMAL);
       if (ce == cudaSuccess && (which == 1 || which == 2)) ce = cap.iter(IK_DUAL);
