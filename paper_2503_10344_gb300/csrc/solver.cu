@@ -720,6 +720,49 @@ static GraphKey graph_key(const Solve& sv, int period) {
   return k;
 }
 
+// ---------------------------------------------------------------- pinned mirrors
+// The pinned host copy of the state that a solve polls.  Allocating and freeing one per solve
+// took 300 us (of 1.65 ms for a 200 x 400 relaxation), so a few outlive their solves: at most
+// kPinnedKept of kPinnedBytes each, handed out under a mutex to one solve at a time and given
+// back when its copies into it are done (a solve that leaves early waits for its stream
+// first); more at once, or larger ones, are allocated and freed as before.
+constexpr size_t kPinnedBytes = 64 << 10;
+constexpr size_t kPinnedKept = 8;
+static std::mutex g_pinned_mu;
+static std::vector<void*>* g_pinned = new std::vector<void*>();
+
+struct Pinned {
+  cudaStream_t s;
+  void* p = nullptr;
+  bool keep = false, idle = false;
+  explicit Pinned(cudaStream_t stream) : s(stream) {}
+  Pinned(const Pinned&) = delete;
+  cudaError_t get(size_t bytes) {
+    keep = bytes <= kPinnedBytes;
+    if (keep) {
+      std::lock_guard<std::mutex> lk(g_pinned_mu);
+      if (!g_pinned->empty()) {
+        p = g_pinned->back();
+        g_pinned->pop_back();
+        return cudaSuccess;
+      }
+    }
+    return cudaHostAlloc(&p, keep ? kPinnedBytes : bytes, cudaHostAllocPortable);
+  }
+  ~Pinned() {
+    if (!p) return;
+    if (!idle && cudaStreamSynchronize(s) != cudaSuccess) keep = false;
+    if (keep) {
+      std::lock_guard<std::mutex> lk(g_pinned_mu);
+      if (g_pinned->size() < kPinnedKept) {
+        g_pinned->push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+};
+
 // ---------------------------------------------------------------- launch-shape autotuner
 // Lanes per row of the two step kernels, chosen by timing: every candidate
 // (2, 4, 8, 16, 32 lanes; the primal kernel's over A^T, then the dual kernel's
@@ -1261,12 +1304,9 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
   } else {
 
   // ---- iteration phase: graph of one check period
-  DevState* hm = nullptr;  // pinned mirror of the first 16 bytes of the state, 2 slots
-  CUDA_TRY(cudaMallocHost(&hm, 2 * sizeof(DevState)));
-  struct HostFree {
-    void* p;
-    ~HostFree() { cudaFreeHost(p); }
-  } hfree{hm};
+  Pinned pinned(s);  // mirror of the first 16 bytes of the state, 2 slots
+  CUDA_TRY(pinned.get(2 * sizeof(DevState)));
+  DevState* hm = (DevState*)pinned.p;
   cudaEvent_t ev[2];
   CUDA_TRY(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
   CUDA_TRY(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
@@ -1420,6 +1460,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     }
   }
   CUDA_TRY(cudaStreamSynchronize(s));  // drain the chunk launched behind the terminating one
+  pinned.idle = true;
   phase("iterations");
   CUDA_TRY(cudaEventRecord(e2, s));
   }  // graph-driven iteration phase
@@ -2220,12 +2261,9 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
       cudaGraphExec_t g;
       ~GFree() { cudaGraphExecDestroy(g); }
     } gfree{ge};
-    DevState* hm = nullptr;
-    CUDA_TRY(cudaMallocHost(&hm, sizeof(DevState) * count));
-    struct HFree {
-      void* p;
-      ~HFree() { cudaFreeHost(p); }
-    } hfree{hm};
+    Pinned pinned(s);
+    CUDA_TRY(pinned.get(sizeof(DevState) * count));
+    DevState* hm = (DevState*)pinned.p;
     const long long max_launches = (p->iter_limit / p->check_period + 2) * 64 + 1024;
     bool forced = false;
     static const int one_flag[2] = {1, 1};
