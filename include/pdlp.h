@@ -143,9 +143,9 @@ typedef struct {
                            (small LPs, such as the 200 x 400 relaxations: no launch per
                            attempt), which copies the LP into shared memory when it fits
                            and otherwise runs the cooperative kernel as one block; 0
-                           (default): the library's choice -- for one LP with float32
-                           iterates that fits, one block or one cooperative kernel with the
-                           LP in the SMs' shared memory (unless lanes_A, lanes_AT, autotune,
+                           (default): the library's choice -- for one LP that fits,
+                           one block or one cooperative kernel with the LP in the SMs'
+                           shared memory (unless lanes_A, lanes_AT, autotune,
                            tiles or halpern ask for the launches), else two kernel launches
                            per attempt.  Same iteration either way.  Batches: 1 runs one cooperative kernel per check
                            period over every LP of the batch (three grid barriers per
@@ -247,7 +247,10 @@ typedef struct {
                              check period stepping from global memory, 3 one block with
                              the LP held in shared memory (persistent = 2 when the matrix,
                              vectors and iterates fit: 76 KB for a 200 x 400 relaxation
-                             with 1,600 nonzeros in float64) */
+                             with 1,600 nonzeros in float64), 4 the LP spread over the
+                             shared memory of all SMs (chosen with persistent = 0 where
+                             it fits; float64 solves that record iterates or the decision
+                             trace run as form 0) */
   double spectral_norm;   /* halpern = 1: L, the power-iteration estimate of ||K~||_2 the
                              step size came from; 0 otherwise */
 } pdlp_result;

@@ -66,19 +66,20 @@ constexpr int kResLong = 64;     // rows longer than this are summed by a warp
 constexpr int kResGatherY = 8;   // gathers in flight per thread: entries of y,
 constexpr int kResGatherX = 4;   // pairs
 constexpr int kResBuckets = 2048;  // buckets the gathers are ordered into
-constexpr int kResReplicas = 16;   // copies of the posted words
+// copies of the posted sums, by the bytes of an iterate element (a float64 slot is three words)
+__host__ __device__ constexpr int res_replicas(int it) { return it == 8 ? 8 : 16; }
 constexpr int kResPoll = 5;      // slots a lane reads at a time (152 SMs: one round)
 constexpr int kResMinStage = 2048;  // nonzeros of A staged at a time at least, if not all are
 
 // Byte offsets of a block's copy of its part of the LP: nt columns with zt nonzeros, na rows
-// with za.  vb: bytes of a matrix value (0: a 0/1 pattern); implicit: per-element step weights
-// are kept.  The stage follows at `bytes`.
+// with za.  it: bytes of an iterate element; vb: of a matrix value (0: a 0/1 pattern); implicit:
+// per-element step weights are kept.  The stage follows at `bytes`.
 struct ResLayout {
   int t_ptr, t_col, t_val, t_lng, a_ptr, a_col, a_val, a_lng;
   int c, l, u, tw, q, sw, kind, x0, x1, y0, y1, sx, sy;
   int bytes;
 };
-__host__ __device__ inline ResLayout res_layout(int nt, int zt, int na, int za, int vb,
+__host__ __device__ inline ResLayout res_layout(int nt, int zt, int na, int za, int it, int vb,
                                                 bool implicit) {
   ResLayout L;
   long long o = 0;
@@ -95,19 +96,19 @@ __host__ __device__ inline ResLayout res_layout(int nt, int zt, int na, int za, 
   L.a_col = take(4LL * za);
   L.a_val = take((long long)vb * za);
   L.a_lng = take(4LL * (za / kResLong + 1));
-  L.c = take(4LL * nt);
-  L.l = take(4LL * nt);
-  L.u = take(4LL * nt);
-  L.tw = take(implicit ? 4LL * nt : 0);
-  L.q = take(4LL * na);
-  L.sw = take(implicit ? 4LL * na : 0);
+  L.c = take((long long)it * nt);
+  L.l = take((long long)it * nt);
+  L.u = take((long long)it * nt);
+  L.tw = take(implicit ? (long long)it * nt : 0);
+  L.q = take((long long)it * na);
+  L.sw = take(implicit ? (long long)it * na : 0);
   L.kind = take(na);
-  L.x0 = take(4LL * nt);
-  L.x1 = take(4LL * nt);
-  L.y0 = take(4LL * na);
-  L.y1 = take(4LL * na);
-  L.sx = take(4LL * nt);
-  L.sy = take(4LL * na);
+  L.x0 = take((long long)it * nt);
+  L.x1 = take((long long)it * nt);
+  L.y0 = take((long long)it * na);
+  L.y1 = take((long long)it * na);
+  L.sx = take((long long)it * nt);
+  L.sy = take((long long)it * na);
   L.bytes = (int)(o < (1LL << 30) ? o : (1LL << 30));
   return L;
 }
@@ -121,9 +122,9 @@ struct ResSizes {
 struct ResPlan {
   int G;                       // blocks (0: the kernel is not used)
   const int *cut_t, *cut_a;    // [G + 1] first column / row of each block
-  ulonglong2* slot;            // [kResReplicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
-  ulonglong2* ex_x;            // [n] published (x', dx), tag
-  unsigned long long* ex_y[2]; // [m] published y, tag
+  void* slot;                  // [res_replicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
+  void* ex_x;                  // [n] published (x', dx), tag
+  void* ex_y[2];               // [m] published y, tag
   int threads, smem;           // per block
   int lanes_t, lanes_a;        // lanes per row of the sums over A^T and A
   int bits_t, bits_a;          // bits of an index of a gather (the rest of its word: the place)
@@ -179,7 +180,8 @@ cudaError_t launch_persist_bf16(int lanes_a, int lanes_t, const IterRaw& r, int 
 cudaError_t launch_persist_pat(int lanes_a, int lanes_t, const IterRaw& r, int max_attempts,
                                int grid, int* grid_out, cudaStream_t s);
 
-// resident step kernel (float32 iterates): the step attempts of a check period
+// resident step kernel: the step attempts of a check period
+cudaError_t launch_resident_fp64(const IterRaw& r, int max_attempts, cudaStream_t s);
 cudaError_t launch_resident_fp32(const IterRaw& r, int max_attempts, cudaStream_t s);
 cudaError_t launch_resident_bf16(const IterRaw& r, int max_attempts, cudaStream_t s);
 cudaError_t launch_resident_pat(const IterRaw& r, int max_attempts, cudaStream_t s);

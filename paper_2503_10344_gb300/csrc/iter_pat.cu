@@ -10,7 +10,7 @@ cudaError_t launch_persist_pat(int lanes_a, int lanes_t, const IterRaw& r, int m
   return launch_persist_t<float, Pattern, true>(lanes_a, lanes_t, r, max_attempts, grid, grid_out, s);
 }
 cudaError_t launch_resident_pat(const IterRaw& r, int max_attempts, cudaStream_t s) {
-  return launch_resident_t<Pattern, true>(r, max_attempts, s);
+  return launch_resident_t<float, Pattern, true>(r, max_attempts, s);
 }
 cudaError_t tile_resident_pat(int form, int* primal_blocks, int* dual_blocks) {
   const cudaError_t e = tile_resident<Pattern, true, false>(form, primal_blocks);

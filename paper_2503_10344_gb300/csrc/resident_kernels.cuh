@@ -1,5 +1,5 @@
-// Step attempts of one LP held in the shared memory of all SMs (rows A4-A7 of the hot path;
-// float32 iterates, LPs of up to ~30 MB).
+// Step attempts of one LP held in the shared memory of all SMs (rows A4-A7 of the hot path; LPs
+// of up to ~30 MB).
 //
 // An LP such as the 50,000 x 200,000 covering LP has 22 MB of step data: it sits in L2, and an
 // attempt of three dependent launches spends its 20 us on launch boundaries and on chains of
@@ -16,7 +16,8 @@
 //   the step decision (A6) by one thread of every block, from the same sums in the same order,
 //   so that all blocks hold bit-identical copies of the step state.
 // There is no grid barrier.  A published entry carries the number of the attempt that made it
-// (y and its tag in 8 bytes, x', dx and theirs in 16: single accesses), a gather reads an entry
+// (in float32 y and its tag in 8 bytes, x', dx and theirs in 16; in float64 every number and its
+// tag in 16: single accesses), a gather reads an entry
 // again until the tag is the one it needs, and the blocks' partial sums travel the same way, one
 // 16-byte word per block.  So a phase starts on each entry as it arrives, without the four trips
 // to L2 that a fence, an arrival, a poll and a fence take (measured: 4,000-5,000 cycles per
@@ -64,25 +65,105 @@ __device__ __forceinline__ unsigned long long pack2(unsigned hi, float lo) {
 }
 __device__ __forceinline__ float low_f(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ unsigned high_u(unsigned long long v) { return (unsigned)(v >> 32); }
+// whether what carries `tag` is older than `want`
+__device__ __forceinline__ bool res_old(unsigned tag, unsigned want) { return (int)(tag - want) < 0; }
 
-// What a gather reads: a published y (tag | y) or pair (dx | x', tag in the second word).
-struct ResY {
+// What is published and gathered: an entry of y, a pair (x', dx), a block's three sums, each
+// with its tag in every word that a single access moves.  float32: y in 8 bytes (tag | y), a
+// pair in 16 (dx | x', tag), the sums in 16; float64: a 16-byte word (value, tag) per number.
+template <typename T> struct ResY;
+template <typename T> struct ResX;
+template <typename T> struct ResS;
+template <> struct ResY<float> {
   using Word = unsigned long long;
   using Acc = float;
   static constexpr int kInFlight = kResGatherY;
   static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u64(p); }
-  static __device__ __forceinline__ unsigned tag(const Word& w) { return high_u(w); }
+  static __device__ __forceinline__ void post(Word* p, float y, unsigned tag) {
+    st_relaxed_u64(p, pack2(tag, y));
+  }
+  static __device__ __forceinline__ bool old(const Word& w, unsigned tag) { return res_old(high_u(w), tag); }
   static __device__ __forceinline__ Acc value(const Word& w) { return low_f(w); }
 };
-struct ResX {
+template <> struct ResX<float> {
   using Word = ulonglong2;
   using Acc = P2<float>;
   static constexpr int kInFlight = kResGatherX;
   static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u128(p); }
-  static __device__ __forceinline__ unsigned tag(const Word& w) { return (unsigned)w.y; }
+  static __device__ __forceinline__ void post(Word* p, float x, float dx, unsigned tag) {
+    st_relaxed_u128(p, ulonglong2{pack2(__float_as_uint(dx), x), tag});
+  }
+  static __device__ __forceinline__ bool old(const Word& w, unsigned tag) {
+    return res_old((unsigned)w.y, tag);
+  }
   static __device__ __forceinline__ Acc value(const Word& w) {
     return Acc{low_f(w.x), __uint_as_float(high_u(w.x))};
   }
+};
+template <> struct ResS<float> {
+  using Word = ulonglong2;
+  static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u128(p); }
+  static __device__ __forceinline__ void post(Word* p, const float (&v)[3], unsigned tag) {
+    st_relaxed_u128(p, ulonglong2{pack2(tag, v[0]), pack2(__float_as_uint(v[2]), v[1])});
+  }
+  static __device__ __forceinline__ bool is(const Word& w, unsigned tag) { return high_u(w.x) == tag; }
+  static __device__ __forceinline__ float value(const Word& w, int k) {
+    return k == 0 ? low_f(w.x) : k == 1 ? low_f(w.y) : __uint_as_float(high_u(w.y));
+  }
+};
+__device__ __forceinline__ ulonglong2 tagged(double v, unsigned tag) {
+  return ulonglong2{(unsigned long long)__double_as_longlong(v), tag};
+}
+__device__ __forceinline__ double untagged(const ulonglong2& w) {
+  return __longlong_as_double((long long)w.x);
+}
+template <> struct ResY<double> {
+  using Word = ulonglong2;
+  using Acc = double;
+  static constexpr int kInFlight = kResGatherY / 2;  // as many bytes
+  static __device__ __forceinline__ Word load(const Word* p) { return ld_relaxed_u128(p); }
+  static __device__ __forceinline__ void post(Word* p, double y, unsigned tag) {
+    st_relaxed_u128(p, tagged(y, tag));
+  }
+  static __device__ __forceinline__ bool old(const Word& w, unsigned tag) {
+    return res_old((unsigned)w.y, tag);
+  }
+  static __device__ __forceinline__ Acc value(const Word& w) { return untagged(w); }
+};
+template <> struct ResX<double> {
+  struct alignas(32) Word {
+    ulonglong2 x, dx;
+  };
+  using Acc = P2<double>;
+  static constexpr int kInFlight = kResGatherX / 2;
+  static __device__ __forceinline__ Word load(const Word* p) {
+    return Word{ld_relaxed_u128(&p->x), ld_relaxed_u128(&p->dx)};
+  }
+  static __device__ __forceinline__ void post(Word* p, double x, double dx, unsigned tag) {
+    st_relaxed_u128(&p->x, tagged(x, tag));
+    st_relaxed_u128(&p->dx, tagged(dx, tag));
+  }
+  static __device__ __forceinline__ bool old(const Word& w, unsigned tag) {
+    return res_old((unsigned)w.x.y, tag) || res_old((unsigned)w.dx.y, tag);
+  }
+  static __device__ __forceinline__ Acc value(const Word& w) {
+    return Acc{untagged(w.x), untagged(w.dx)};
+  }
+};
+template <> struct ResS<double> {
+  struct Word {
+    ulonglong2 v[3];
+  };
+  static __device__ __forceinline__ Word load(const Word* p) {
+    return Word{{ld_relaxed_u128(p->v), ld_relaxed_u128(p->v + 1), ld_relaxed_u128(p->v + 2)}};
+  }
+  static __device__ __forceinline__ void post(Word* p, const double (&v)[3], unsigned tag) {
+    for (int k = 0; k < 3; ++k) st_relaxed_u128(p->v + k, tagged(v[k], tag));
+  }
+  static __device__ __forceinline__ bool is(const Word& w, unsigned tag) {
+    return (unsigned)w.v[0].y == tag && (unsigned)w.v[1].y == tag && (unsigned)w.v[2].y == tag;
+  }
+  static __device__ __forceinline__ double value(const Word& w, int k) { return untagged(w.v[k]); }
 };
 
 // a bounded wait: false once the limit has passed or another block has given up
@@ -108,33 +189,52 @@ __device__ __forceinline__ float div_pos(float n, float d) {
   return fmaf(fmaf(-q, d, n), r, q);
 }
 
-// This block's three sums (lane-uniform) posted to every replica under `tag`, and the sums over
-// all blocks in slot order per lane, then a fixed shuffle tree.  Called by one whole warp.
-// (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.)
-__device__ __forceinline__ bool res_sums(DevState* st, ulonglong2* slot, int G, unsigned tag,
-                                         int limit, float (&sum)[3]) {
-  const int lane = threadIdx.x & 31, b = blockIdx.x;
-  if (lane < kResReplicas) {
-    const ulonglong2 w{pack2(tag, sum[0]), pack2(__float_as_uint(sum[2]), sum[1])};
-    st_relaxed_u128(slot + (size_t)lane * G + b, w);
+// Sum over a warp whose lanes other than the multiples of `step` (a power of two) below `used`
+// hold zeros, in every lane that is such a multiple (lane 0 among them): the levels that would add
+// zeros only are left out, and all of them where every lane holds zero (rows that did not move,
+// warps without rows).  In float64 a level costs a warp some 16 cycles of the SM's one pipe; in
+// float32 the tests would cost more than the levels, and all are added.
+template <typename T>
+__device__ __forceinline__ T res_warp_sum(T v, int step, int used) {
+  if constexpr (std::is_same<T, float>::value) return group_sum<32>(v);
+  if (!__any_sync(0xffffffffu, v != (T)0)) return (T)0;
+  for (int o = 16; o >= step; o >>= 1) {
+    const T w = __shfl_xor_sync(0xffffffffu, v, o);
+    if (o < used) v += w;
   }
-  const ulonglong2* mine = slot + (size_t)(b % kResReplicas) * G;
-  bool ok = true;
-  sum[0] = sum[1] = sum[2] = 0.f;
-  ResWait wait{st, limit, 0};
-  for (int b0 = 0; b0 < G; b0 += 32 * kResPoll) {
-    ulonglong2 w[kResPoll];
+  return v;
+}
+
+// This block's three sums (of lane 0) posted to every replica under `tag`, and the sums over
+// all blocks in slot order per lane, then a fixed shuffle tree (in lane 0).  Called by one whole warp.
+// (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.)
+template <typename T>
+__device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* slot, int G,
+                                         unsigned tag, int limit, T (&sum)[3]) {
+  using S = ResS<T>;
+  constexpr int reps = res_replicas((int)sizeof(T)), kPoll = sizeof(T) == 8 ? 2 : kResPoll;
+  const int lane = threadIdx.x & 31, b = blockIdx.x;
+  if constexpr (std::is_same<T, double>::value)
 #pragma unroll
-    for (int i = 0; i < kResPoll; ++i)
-      if (b0 + i * 32 + lane < G) w[i] = ld_relaxed_u128(mine + b0 + i * 32 + lane);
+    for (int k = 0; k < 3; ++k) sum[k] = __shfl_sync(0xffffffffu, sum[k], 0);
+  if (lane < reps) S::post(slot + (size_t)lane * G + b, sum, tag);
+  const typename S::Word* mine = slot + (size_t)(b % reps) * G;
+  bool ok = true;
+  sum[0] = sum[1] = sum[2] = (T)0;
+  ResWait wait{st, limit, 0};
+  for (int b0 = 0; b0 < G; b0 += 32 * kPoll) {
+    typename S::Word w[kPoll];
+#pragma unroll
+    for (int i = 0; i < kPoll; ++i)
+      if (b0 + i * 32 + lane < G) w[i] = S::load(mine + b0 + i * 32 + lane);
     bool miss = true;
     while (miss) {
       miss = false;
 #pragma unroll
-      for (int i = 0; i < kResPoll; ++i)
-        if (b0 + i * 32 + lane < G && high_u(w[i].x) != tag) {
+      for (int i = 0; i < kPoll; ++i)
+        if (b0 + i * 32 + lane < G && !S::is(w[i], tag)) {
           miss = true;
-          w[i] = ld_relaxed_u128(mine + b0 + i * 32 + lane);
+          w[i] = S::load(mine + b0 + i * 32 + lane);
         }
       if (miss && !wait.more()) {
         ok = false;
@@ -142,18 +242,15 @@ __device__ __forceinline__ bool res_sums(DevState* st, ulonglong2* slot, int G, 
       }
     }
 #pragma unroll
-    for (int i = 0; i < kResPoll; ++i)
+    for (int i = 0; i < kPoll; ++i)
       if (b0 + i * 32 + lane < G) {
-        sum[0] += low_f(w[i].x);
-        sum[1] += low_f(w[i].y);
-        sum[2] += __uint_as_float(high_u(w[i].y));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum[k] += S::value(w[i], k);
       }
   }
   ok = __all_sync(0xffffffffu, ok);
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+  for (int k = 0; k < 3; ++k) sum[k] = res_warp_sum<T>(sum[k], 1, G);
   return ok;
 }
 
@@ -167,10 +264,10 @@ struct ResSide {
   int rows, nlong, bits, cap;
 };
 
-template <typename V>
-__device__ __forceinline__ float res_val(const V* v, int p) {
-  if constexpr (std::is_same<V, Pattern>::value) return 1.f;
-  else if constexpr (std::is_same<V, float>::value) return v[p];
+template <typename T, typename V>
+__device__ __forceinline__ T res_val(const V* v, int p) {
+  if constexpr (std::is_same<V, Pattern>::value) return (T)1;
+  else if constexpr (std::is_same<V, T>::value) return v[p];
   else return __bfloat162float(v[p]);
 }
 
@@ -228,17 +325,17 @@ __device__ __forceinline__ void res_sort_keys(const int* __restrict__ col, int n
 
 // Sums over the staged entries of rows [ra, rb) of the chunk that starts at nonzero p0, and
 // their epilogues: LANES lanes per row, then a warp per long row.
-template <int LANES, typename Acc, typename V, typename Fin>
+template <int LANES, typename T, typename Acc, typename V, typename Fin>
 __device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, int p0, int ra,
                                          int rb, Fin fin) {
-  const int lane = threadIdx.x & (LANES - 1), T = blockDim.x;
+  const int lane = threadIdx.x & (LANES - 1), NT = blockDim.x;
   auto add = [&](Acc& acc, int p) {
-    const float v = res_val<V>(s.val, p);
+    const T v = res_val<T, V>(s.val, p);
     const Acc t = stage[p - p0];
-    if constexpr (std::is_same<Acc, float>::value) acc += v * t;
+    if constexpr (std::is_same<Acc, T>::value) acc += v * t;
     else acc += Acc{v * t.a, v * t.b};
   };
-  for (int r = ra + (int)threadIdx.x / LANES; r < rb; r += T / LANES) {
+  for (int r = ra + (int)threadIdx.x / LANES; r < rb; r += NT / LANES) {
     const int b = s.ptr[r], e = s.ptr[r + 1];
     if (e - b > kResLong) continue;  // uniform within the group
     Acc acc{};
@@ -248,7 +345,7 @@ __device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, 
     if (lane == 0) fin(r, acc);
   }
   const int wl = threadIdx.x & 31;
-  for (int k = threadIdx.x >> 5; k < s.nlong; k += T >> 5) {
+  for (int k = threadIdx.x >> 5; k < s.nlong; k += NT >> 5) {
     const int r = s.lng[k];
     if (r < ra || r >= rb) continue;
     const int b = s.ptr[r], e = s.ptr[r + 1];
@@ -260,15 +357,15 @@ __device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, 
   }
 }
 
-template <typename Acc, typename V, typename Fin>
+template <typename T, typename Acc, typename V, typename Fin>
 __device__ __forceinline__ void res_rows_lanes(int lanes, const ResSide<V>& s, const Acc* stage,
                                                int p0, int ra, int rb, Fin fin) {
   switch (lanes) {
-    case 1: return res_rows<1>(s, stage, p0, ra, rb, fin);
-    case 2: return res_rows<2>(s, stage, p0, ra, rb, fin);
-    case 4: return res_rows<4>(s, stage, p0, ra, rb, fin);
-    case 8: return res_rows<8>(s, stage, p0, ra, rb, fin);
-    default: return res_rows<16>(s, stage, p0, ra, rb, fin);
+    case 1: return res_rows<1, T>(s, stage, p0, ra, rb, fin);
+    case 2: return res_rows<2, T>(s, stage, p0, ra, rb, fin);
+    case 4: return res_rows<4, T>(s, stage, p0, ra, rb, fin);
+    case 8: return res_rows<8, T>(s, stage, p0, ra, rb, fin);
+    default: return res_rows<16, T>(s, stage, p0, ra, rb, fin);
   }
 }
 
@@ -296,7 +393,7 @@ __device__ __forceinline__ bool res_gather(const ResSide<V>& s, int p0, int n,
       miss = false;
 #pragma unroll
       for (int k = 0; k < U; ++k)
-        if (i0 + k * nt < n && (int)(E::tag(w[k]) - tag) < 0) {
+        if (i0 + k * nt < n && E::old(w[k], tag)) {
           miss = true;
           w[k] = E::load(from + (c[k] & mask));
         }
@@ -311,7 +408,7 @@ __device__ __forceinline__ bool res_gather(const ResSide<V>& s, int p0, int n,
 
 // A side's product: chunk by chunk the entries its rows need, then the rows' sums.  The first
 // chunk may have been gathered ahead (`ahead`).
-template <typename E, typename V, typename Fin>
+template <typename T, typename E, typename V, typename Fin>
 __device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
                                             const typename E::Word* from, unsigned tag,
                                             typename E::Acc* stage, bool ahead, ResWait wait,
@@ -324,47 +421,62 @@ __device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
       if (!res_gather<E>(s, p0, s.ptr[rb] - p0, from, tag, stage, threadIdx.x, blockDim.x, wait))
         *fail = 1;
     __syncthreads();
-    res_rows_lanes<typename E::Acc>(lanes, s, stage, p0, ra, rb, fin);
+    res_rows_lanes<T, typename E::Acc>(lanes, s, stage, p0, ra, rb, fin);
     ra = rb;
   }
 }
 
-// The step decision (decide_step in float32, the same operations) in two halves: what the next
-// attempt reads, which every thread of the block waits for, and the rest of the state, which
+// The step decision (decide_step, the same operations in the iterate type) in two halves: what the
+// next attempt reads, which every thread of the block waits for, and the rest of the state, which
 // the deciding thread writes while the others go on.
+template <typename T>
 struct ResDecision {
-  float eta, eta_bar, eta_next;
+  T eta, eta_bar, eta_next;
   bool accept;
 };
-__device__ __forceinline__ ResDecision res_decide(DevState* st, float dx2, float dy2, float dkd,
-                                                  float fd, float fi, int& left) {
-  ResDecision r{st->eta_f, INFINITY, st->eta_f, true};
+template <typename T>
+__device__ __forceinline__ ResDecision<T> res_decide(DevState* st, T dx2, T dy2, T dkd, T fd, T fi,
+                                                     int& left) {
+  constexpr bool F64 = std::is_same<T, double>::value;
+  const T eta = F64 ? (T)st->eta : (T)st->eta_f;
+  ResDecision<T> r{eta, (T)INFINITY, eta, true};
   if (!isfinite(dx2) || !isfinite(dy2) || !isfinite(dkd)) {
     st->status = 4;  // PDLP_NUMERICAL
     return r;
   }
-  const float om = st->omega_f, iom = st->inv_omega_f;
+  const T om = F64 ? (T)st->omega : (T)st->omega_f, iom = F64 ? (T)0 : (T)st->inv_omega_f;
   if (st->adaptive || st->tr_cap > 0) {  // (a fixed step needs the bound for the trace alone)
-    const float den = 2.f * fabsf(dkd);
-    r.eta_bar = den > 0.f ? (om * dx2 + dy2 * iom) / den : INFINITY;
+    const T den = (T)2 * fabs(dkd);
+    const T num = F64 ? om * dx2 + dy2 / om : om * dx2 + dy2 * iom;
+    r.eta_bar = den > (T)0 ? num / den : (T)INFINITY;
   }
   if (st->adaptive) {
-    r.eta_next = fminf(fd * r.eta_bar, fi * r.eta);
+    r.eta_next = fmin(fd * r.eta_bar, fi * r.eta);
     r.accept = !(r.eta > r.eta_bar);
   }
   if (r.accept) {
     st->cur ^= 1;
-    st->pw_f = r.eta;
     if (--left == 0) st->check_due = 1;
-  } else {
-    st->pw_f = 0.f;
   }
-  st->eta_f = r.eta_next;
-  st->tau_f = r.eta_next * iom;
-  st->sigma_f = r.eta_next * om;
+  const T pw = r.accept ? r.eta : (T)0;
+  if constexpr (F64) {
+    st->pending_w = pw;
+    st->pw_f = (float)pw;
+    if (r.eta_next != r.eta) {  // (else the quotient that is there already)
+      st->eta = r.eta_next;
+      st->tau_d = r.eta_next / om;
+      st->sigma_d = r.eta_next * om;
+    }
+  } else {
+    st->pw_f = pw;
+    st->eta_f = r.eta_next;
+    st->tau_f = r.eta_next * iom;
+    st->sigma_f = r.eta_next * om;
+  }
   return r;
 }
-__device__ __forceinline__ void res_record(DevState* st, const ResDecision& r) {
+template <typename T>
+__device__ __forceinline__ void res_record(DevState* st, const ResDecision<T>& r) {
   const long long t = st->attempts;
   st->attempts = t + 1;
   if (st->status == 4) return;
@@ -374,32 +486,34 @@ __device__ __forceinline__ void res_record(DevState* st, const ResDecision& r) {
     st->tr_accepted[t] = r.accept ? 1 : 0;
   }
   if (r.accept) {
-    st->pending_w = (double)r.eta;
     st->sum_w += (double)r.eta;
     st->iters += 1;
-  } else {
-    st->pending_w = 0.0;
   }
-  st->eta = (double)r.eta_next;
+  if constexpr (std::is_same<T, float>::value) {
+    st->pending_w = r.accept ? (double)r.eta : 0.0;
+    st->eta = (double)r.eta_next;
+  }
 }
 
-template <typename V, bool IMPLICIT>
-__global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d, ResPlan R,
+template <typename T, typename V, bool IMPLICIT>
+__global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, ResPlan R,
                                                            int max_attempts) {
+  using EY = ResY<T>;
+  using EX = ResX<T>;
   constexpr bool VALS = !std::is_same<V, Pattern>::value;
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ DevState ls;
-  __shared__ float red[3][32];  // the warps' sums (0 beyond the block's warps)
+  __shared__ T red[3][32];  // the warps' sums (0 beyond the block's warps)
   __shared__ int nlong[2], stop, fail;
   DevState* gst = d.st;
-  const int tid = threadIdx.x, T = blockDim.x, G = R.G, b = blockIdx.x;
+  const int tid = threadIdx.x, NT = blockDim.x, G = R.G, b = blockIdx.x;
   if (tid == 0) {
     ls = *gst;
     if (b != 0) ls.tr_cap = 0;  // one block writes the trace
     stop = (ls.status != 0 || ls.check_due) ? 1 : 0;
     fail = 0;
   }
-  if (tid < 32) red[0][tid] = red[1][tid] = red[2][tid] = 0.f;
+  if (tid < 32) red[0][tid] = red[1][tid] = red[2][tid] = (T)0;
   __syncthreads();
   if (stop) return;
   // ---- the block's columns [t0, t1) and rows [a0, a1)
@@ -407,7 +521,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
   const int nt = t1 - t0, na = a1 - a0;
   const int tz0 = __ldg(d.t_ptr + t0), az0 = __ldg(d.a_ptr + a0);
   const int tz = __ldg(d.t_ptr + t1) - tz0, az = __ldg(d.a_ptr + a1) - az0;
-  const ResLayout L = res_layout(nt, tz, na, az, VALS ? (int)sizeof(V) : 0, IMPLICIT);
+  const ResLayout L = res_layout(nt, tz, na, az, (int)sizeof(T), VALS ? (int)sizeof(V) : 0, IMPLICIT);
   int* tp = (int*)(sm + L.t_ptr);
   unsigned* tk = (unsigned*)(sm + L.t_col);
   V* tv = VALS ? (V*)(sm + L.t_val) : nullptr;
@@ -416,35 +530,37 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
   unsigned* ak = (unsigned*)(sm + L.a_col);
   V* av = VALS ? (V*)(sm + L.a_val) : nullptr;
   int* al = (int*)(sm + L.a_lng);
-  float* c = (float*)(sm + L.c);
-  float* l = (float*)(sm + L.l);
-  float* u = (float*)(sm + L.u);
-  float* tw = IMPLICIT ? (float*)(sm + L.tw) : nullptr;
-  float* q = (float*)(sm + L.q);
-  float* sw = IMPLICIT ? (float*)(sm + L.sw) : nullptr;
+  T* c = (T*)(sm + L.c);
+  T* l = (T*)(sm + L.l);
+  T* u = (T*)(sm + L.u);
+  T* tw = IMPLICIT ? (T*)(sm + L.tw) : nullptr;
+  T* q = (T*)(sm + L.q);
+  T* sw = IMPLICIT ? (T*)(sm + L.sw) : nullptr;
   unsigned char* kind = sm + L.kind;
-  float* xs[2] = {(float*)(sm + L.x0), (float*)(sm + L.x1)};
-  float* ys[2] = {(float*)(sm + L.y0), (float*)(sm + L.y1)};
-  float* sx = (float*)(sm + L.sx);
-  float* sy = (float*)(sm + L.sy);
-  P2<float>* stage2 = (P2<float>*)(sm + L.bytes);
-  float* stage1 = (float*)(sm + L.bytes);
+  T* xs[2] = {(T*)(sm + L.x0), (T*)(sm + L.x1)};
+  T* ys[2] = {(T*)(sm + L.y0), (T*)(sm + L.y1)};
+  T* sx = (T*)(sm + L.sx);
+  T* sy = (T*)(sm + L.sy);
+  P2<T>* stage2 = (P2<T>*)(sm + L.bytes);
+  T* stage1 = (T*)(sm + L.bytes);
+  typename EX::Word* const ex_x = (typename EX::Word*)R.ex_x;
+  auto ex_y = [&](int k) { return (typename EY::Word*)R.ex_y[k]; };
   // ---- copy in (iterates with ordinary loads: the KKT block of the same graph wrote them);
   // the y of this launch is published under a tag of its own
-  for (int i = tid; i <= nt; i += T) tp[i] = __ldg(d.t_ptr + t0 + i) - tz0;
-  for (int i = tid; i <= na; i += T) ap[i] = __ldg(d.a_ptr + a0 + i) - az0;
+  for (int i = tid; i <= nt; i += NT) tp[i] = __ldg(d.t_ptr + t0 + i) - tz0;
+  for (int i = tid; i <= na; i += NT) ap[i] = __ldg(d.a_ptr + a0 + i) - az0;
   const int cur0 = ls.cur;
   const unsigned tag0 = 2u * (unsigned)ls.attempts;
-  for (int i = tid; i < na; i += T) {
-    const float y = d.y[cur0][a0 + i];
-    st_relaxed_u64(R.ex_y[cur0] + a0 + i, pack2(tag0 + 1u, y));
+  for (int i = tid; i < na; i += NT) {
+    const T y = d.y[cur0][a0 + i];
+    EY::post(ex_y(cur0) + a0 + i, y, tag0 + 1u);
     ys[cur0][i] = y;
     q[i] = __ldg(d.q + a0 + i);
     if constexpr (IMPLICIT) sw[i] = __ldg(d.sw + a0 + i);
     kind[i] = __ldg(d.row_kind + a0 + i);
     sy[i] = d.sum_y[a0 + i];
   }
-  for (int j = tid; j < nt; j += T) {
+  for (int j = tid; j < nt; j += NT) {
     c[j] = __ldg(d.c + t0 + j);
     l[j] = __ldg(d.l + t0 + j);
     u[j] = __ldg(d.u + t0 + j);
@@ -453,8 +569,8 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
     sx[j] = d.sum_x[t0 + j];
   }
   if constexpr (VALS) {
-    for (int p = tid; p < tz; p += T) tv[p] = d.t_val[tz0 + p];
-    for (int p = tid; p < az; p += T) av[p] = d.a_val[az0 + p];
+    for (int p = tid; p < tz; p += NT) tv[p] = d.t_val[tz0 + p];
+    for (int p = tid; p < az; p += NT) av[p] = d.a_val[az0 + p];
   }
   __syncthreads();
   // the gathers of every chunk, ordered
@@ -495,61 +611,63 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
   const ResSide<V> sa{ap, ak, av, al, na, nlong[1], R.bits_a, R.cap_a};
   const int ahead_n = nt ? tp[res_chunk_end(tp, nt, R.cap_t, 0)] : 0;  // the first chunk of st
   const ResWait wait{gst, (int)ls.spin_limit, 0};
-  ResDecision dec{};
+  ResDecision<T> dec{};
   unsigned ytag = tag0 + 1u;
   bool ahead = false;  // the first chunk of the next primal step is staged
   for (int att = 0; att < max_attempts; ++att) {
     const int cur = ls.cur;
-    const float pw = ls.pw_f, tau = ls.tau_f, sigma = ls.sigma_f;
+    const T pw = StepT<T>::pw(&ls), tau = StepT<T>::tau(&ls), sigma = StepT<T>::sigma(&ls);
     const unsigned tag = tag0 + 2u * (unsigned)(att + 1);
-    float fd = 0.f, fi = 0.f;
+    T fd = 0, fi = 0;
     if (tid == 0) {
       if (att > 0) res_record(&ls, dec);  // of the attempt before
       step_factors(&ls, ls.attempts + 1, &fd, &fi);
     }
     // ---- A4: primal step over the block's columns
     {
-      const float* xo = xs[cur];
-      float* xn = xs[cur ^ 1];
-      float dx2 = 0.f;
-      auto fin = [&](int j, float aty) {
-        const float x = xo[j];
-        const float w = IMPLICIT ? tw[j] : 1.f;
-        const float step = IMPLICIT ? tau * w : tau;
-        const float xv = clampv(x - step * (c[j] - aty), l[j], u[j]);
-        const float dd = xv - x;
+      const T* xo = xs[cur];
+      T* xn = xs[cur ^ 1];
+      T dx2 = 0;
+      auto fin = [&](int j, T aty) {
+        const T x = xo[j];
+        const T w = IMPLICIT ? tw[j] : (T)1;
+        const T step = IMPLICIT ? tau * w : tau;
+        const T xv = clampv(x - step * (c[j] - aty), l[j], u[j]);
+        const T dd = xv - x;
         xn[j] = xv;
-        st_relaxed_u128(R.ex_x + t0 + j, ulonglong2{pack2(__float_as_uint(dd), xv), tag});
-        if (pw != 0.f) sx[j] += pw * x;  // A7: add the iterate whose weight is pending
-        dx2 += IMPLICIT ? div_pos(dd * dd, w) : dd * dd;
+        EX::post(ex_x + t0 + j, xv, dd, tag);
+        if (pw != (T)0) sx[j] += pw * x;  // A7: add the iterate whose weight is pending
+        if constexpr (IMPLICIT) dx2 += div_pos(dd * dd, w);
+        else dx2 += dd * dd;
       };
-      res_product<ResY>(R.lanes_t, st, R.ex_y[cur], ytag, stage1, ahead, wait, &fail, fin);
-      dx2 = group_sum<32>(dx2);
+      res_product<T, EY>(R.lanes_t, st, ex_y(cur), ytag, stage1, ahead, wait, &fail, fin);
+      dx2 = res_warp_sum<T>(dx2, R.lanes_t, 32);
       if ((tid & 31) == 0) red[0][tid >> 5] = dx2;
     }
     __syncthreads();  // the stage is free
     // ---- A5: dual step over the block's rows
     {
-      const float* yo = ys[cur];
-      float* yn = ys[cur ^ 1];
-      unsigned long long* gy = R.ex_y[cur ^ 1];
-      float dy2 = 0.f, dkd = 0.f;
-      auto fin = [&](int i, P2<float> acc) {  // acc.a = (K x')_i, acc.b = (K dx)_i
-        const float y = yo[i];
-        const float w = IMPLICIT ? sw[i] : 1.f;
-        const float step = IMPLICIT ? sigma * w : sigma;
-        float yv = y + step * (q[i] - (acc.a + acc.b));
-        if (kind[i] != 1) yv = fmaxf(yv, 0.f);
-        st_relaxed_u64(gy + a0 + i, pack2(tag, yv));
+      const T* yo = ys[cur];
+      T* yn = ys[cur ^ 1];
+      typename EY::Word* gy = ex_y(cur ^ 1);
+      T dy2 = 0, dkd = 0;
+      auto fin = [&](int i, P2<T> acc) {  // acc.a = (K x')_i, acc.b = (K dx)_i
+        const T y = yo[i];
+        const T w = IMPLICIT ? sw[i] : (T)1;
+        const T step = IMPLICIT ? sigma * w : sigma;
+        T yv = y + step * (q[i] - (acc.a + acc.b));
+        if (kind[i] != 1) yv = maxv(yv, (T)0);
+        EY::post(gy + a0 + i, yv, tag);
         yn[i] = yv;
-        if (pw != 0.f) sy[i] += pw * y;
-        const float dd = yv - y;
-        dy2 += IMPLICIT ? div_pos(dd * dd, w) : dd * dd;
+        if (pw != (T)0) sy[i] += pw * y;
+        const T dd = yv - y;
+        if constexpr (IMPLICIT) dy2 += div_pos(dd * dd, w);
+        else dy2 += dd * dd;
         dkd += dd * acc.b;
       };
-      res_product<ResX>(R.lanes_a, sa, R.ex_x, tag, stage2, false, wait, &fail, fin);
-      dy2 = group_sum<32>(dy2);
-      dkd = group_sum<32>(dkd);
+      res_product<T, EX>(R.lanes_a, sa, ex_x, tag, stage2, false, wait, &fail, fin);
+      dy2 = res_warp_sum<T>(dy2, R.lanes_a, 32);
+      dkd = res_warp_sum<T>(dkd, R.lanes_a, 32);
       if ((tid & 31) == 0) {
         red[1][tid >> 5] = dy2;
         red[2][tid >> 5] = dkd;
@@ -557,17 +675,17 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
     }
     __syncthreads();  // the stage is free, the warps' sums are there
     if (tid < 32) {
-      float s[3];
+      T s[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) s[k] = group_sum<32>(red[k][tid]);
+      for (int k = 0; k < 3; ++k) s[k] = res_warp_sum<T>(red[k][tid], 1, NT >> 5);
       bool ok = fail == 0;
-      if (G > 1) ok = res_sums(gst, R.slot, G, tag, wait.limit, s) && ok;
+      if (G > 1) ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, G, tag, wait.limit, s) && ok;
       // ---- A6: the same decision in every block
       if (tid == 0) {
-        dec = res_decide(&ls, s[0], s[1], s[2], fd, fi, left);
+        dec = res_decide<T>(&ls, s[0], s[1], s[2], fd, fi, left);
         stop = !ok ? 2 : (ls.status != 0 || ls.check_due) ? 1 : 0;
       }
-    } else if (!res_gather<ResY>(st, 0, ahead_n, R.ex_y[cur ^ 1], tag, stage1, tid - 32, T - 32,
+    } else if (!res_gather<EY>(st, 0, ahead_n, ex_y(cur ^ 1), tag, stage1, tid - 32, NT - 32,
                                  wait)) {
       fail = 1;
     }
@@ -587,11 +705,14 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<float, V> d,
   if (tid == 0 && max_attempts > 0) res_record(&ls, dec);  // of the last attempt
   // ---- copy out: the iterate (its step is not needed any more) and the running sums
   const int cur = ls.cur;
-  for (int j = tid; j < nt; j += T) {
-    d.x[cur][t0 + j] = make_float2(xs[cur][j], 0.f);
+  for (int j = tid; j < nt; j += NT) {
+    vec2_t<T> o;
+    o.x = xs[cur][j];
+    o.y = (T)0;
+    d.x[cur][t0 + j] = o;
     d.sum_x[t0 + j] = sx[j];
   }
-  for (int i = tid; i < na; i += T) {
+  for (int i = tid; i < na; i += NT) {
     d.y[cur][a0 + i] = ys[cur][i];
     d.sum_y[a0 + i] = sy[i];
   }

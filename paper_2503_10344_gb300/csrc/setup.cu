@@ -1214,8 +1214,8 @@ cudaError_t setup_len_order(const int* ptr, int rows, int* ord, cudaStream_t s) 
 constexpr int kResRowWeight = 4;
 __global__ void __launch_bounds__(kBlock) k_res_plan(int m, int n, long long nnz,
                                                      const int* a_ptr, const int* t_ptr, int G,
-                                                     int vb, int implicit, int* cut_t, int* cut_a,
-                                                     ResSizes* sizes) {
+                                                     int it, int vb, int implicit, int* cut_t,
+                                                     int* cut_a, ResSizes* sizes) {
   int longest = 0;
   const long long stride = (long long)gridDim.x * kBlock;
   for (long long i = (long long)blockIdx.x * kBlock + threadIdx.x; i < (long long)m + n;
@@ -1249,15 +1249,15 @@ __global__ void __launch_bounds__(kBlock) k_res_plan(int m, int n, long long nnz
     atomicMax(&sizes->t_nnz, zt);
     atomicMax(&sizes->a_rows, na);
     atomicMax(&sizes->a_nnz, za);
-    atomicMax(&sizes->bytes, res_layout(nt, zt, na, za, vb, implicit != 0).bytes);
+    atomicMax(&sizes->bytes, res_layout(nt, zt, na, za, it, vb, implicit != 0).bytes);
   }
 }
 
-cudaError_t setup_res_plan(int m, int n, int nnz, const int* a_ptr, const int* t_ptr, int G, int vb,
-                           bool implicit, int* cut_t, int* cut_a, ResSizes* sizes, cudaStream_t s) {
+cudaError_t setup_res_plan(int m, int n, int nnz, const int* a_ptr, const int* t_ptr, int G, int it,
+                           int vb, bool implicit, int* cut_t, int* cut_a, ResSizes* sizes, cudaStream_t s) {
   RET(cudaMemsetAsync(sizes, 0, sizeof(ResSizes), s));
   k_res_plan<<<grid_for((long long)m + n, device_sm_count()), kBlock, 0, s>>>(
-      m, n, nnz, a_ptr, t_ptr, G, vb, implicit ? 1 : 0, cut_t, cut_a, sizes);
+      m, n, nnz, a_ptr, t_ptr, G, it, vb, implicit ? 1 : 0, cut_t, cut_a, sizes);
   return cudaGetLastError();
 }
 

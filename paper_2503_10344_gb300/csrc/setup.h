@@ -103,8 +103,8 @@ cudaError_t setup_power_norm(const PowIn& q, int iters, double* u, double* w, do
 
 // The parts of a resident step kernel of G blocks (G < kBlock): cut_t[G + 1], cut_a[G + 1] and
 // the sizes they come to (device); vb, implicit as in res_layout.
-cudaError_t setup_res_plan(int m, int n, int nnz, const int* a_ptr, const int* t_ptr, int G, int vb,
-                           bool implicit, int* cut_t, int* cut_a, ResSizes* sizes, cudaStream_t s);
+cudaError_t setup_res_plan(int m, int n, int nnz, const int* a_ptr, const int* t_ptr, int G, int it,
+                           int vb, bool implicit, int* cut_t, int* cut_a, ResSizes* sizes, cudaStream_t s);
 
 // Bound-objective rescaling of the iteration vectors and the start point, with the
 // factors beta (right-hand side, bounds, x) and gamma (objective, y) folded into the

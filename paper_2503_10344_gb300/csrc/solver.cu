@@ -157,8 +157,8 @@ static size_t carve(Arena& ar, Bufs& b, int m, int n, long long nnz, int precisi
   b.c_it = ar.take(eb * N);
   b.l_it = ar.take(eb * N);
   b.u_it = ar.take(eb * N);
-  b.tw = ar.take(eb * N);
   b.q_it = ar.take(eb * M);
+  b.tw = ar.take(eb * N);
   b.sw = ar.take(eb * M);
   for (int k = 0; k < 2; ++k) {
     b.x[k] = ar.take(2 * eb * N);  // (x_j, dx_j) pairs
@@ -295,6 +295,7 @@ struct Solve {
     int g = 0;
     if (ir.res.G > 0) {
       switch (mode) {
+        case MODE_FP64: return launch_resident_fp64(ir, max_attempts, s);
         case MODE_FP32: return launch_resident_fp32(ir, max_attempts, s);
         case MODE_BF16: return launch_resident_bf16(ir, max_attempts, s);
         default: return launch_resident_pat(ir, max_attempts, s);
@@ -446,6 +447,60 @@ static int check_inputs(const pdlp_csr* A, const void* b, const void* sense, con
   return PDLP_OK;
 }
 
+// Buffers of the resident step kernel in scratch that is free once the setup is done (the
+// workspace does not grow for them): each array in the first of `regions` with room for it.
+struct Region {
+  void* base;
+  size_t bytes;
+};
+struct ResBufs {
+  void *ex_x = nullptr, *ex_y[2] = {nullptr, nullptr}, *slot = nullptr;
+  int *cut_t = nullptr, *cut_a = nullptr;
+  ResSizes* sizes = nullptr;
+  size_t x_bytes = 0, y_bytes = 0, slot_bytes = 0;
+  bool ok = false;  // all of them found room
+  // `it`: bytes of an iterate element (the words published: resident_kernels.cuh)
+  bool place(const Region* regions, int count, int G, long long m, long long n, int it) {
+    Arena ar[4];
+    for (int k = 0; k < count; ++k) ar[k] = Arena{(char*)regions[k].base, 0};
+    ok = true;
+    auto take = [&](size_t bytes) -> void* {
+      for (int k = 0; k < count; ++k) {
+        Arena a = ar[k];
+        void* p = a.take(bytes);
+        if (a.off <= regions[k].bytes) {
+          ar[k] = a;
+          return p;
+        }
+      }
+      ok = false;
+      return nullptr;
+    };
+    x_bytes = (it == 8 ? 32 : 16) * (size_t)n;
+    y_bytes = (it == 8 ? 16 : 8) * (size_t)m;
+    slot_bytes = (it == 8 ? 48 : 16) * (size_t)res_replicas(it) * G;
+    slot = take(slot_bytes);
+    ex_x = take(x_bytes);
+    for (void*& y : ex_y) y = take(y_bytes);
+    cut_t = (int*)take(4 * ((size_t)G + 1));
+    cut_a = (int*)take(4 * ((size_t)G + 1));
+    sizes = (ResSizes*)take(sizeof(ResSizes));
+    return ok;
+  }
+  // zeros (no tag) in everything published; neighbours in one go
+  cudaError_t clear(cudaStream_t s) const {
+    char* p[4] = {(char*)slot, (char*)ex_x, (char*)ex_y[0], (char*)ex_y[1]};
+    const size_t b[4] = {slot_bytes, x_bytes, y_bytes, y_bytes};
+    for (int k = 0; k < 4;) {
+      char *from = p[k], *to = p[k] + b[k];
+      for (++k; k < 4 && p[k] >= to && p[k] - to < 256; ++k) to = p[k] + b[k];
+      const cudaError_t e = cudaMemsetAsync(from, 0, (size_t)(to - from), s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+};
+
 // Kernel timing request (pdlp_time_kernels): after the setup of a solve, each
 // fused kernel is launched `reps` times back to back from a CUDA graph.
 struct TimingReq {
@@ -456,7 +511,8 @@ struct TimingReq {
 };
 
 static int time_kernels_after_setup(Solve& sv, DevState* st, int mode, long long nnz,
-                                    const TimingReq& tq, int count);
+                                    const TimingReq& tq, int count,
+                                    const ResBufs* rb = nullptr);
 
 // Products of the device setup of one LP (rows A0-A3) into the buffers of a Bufs.
 struct SetupOut {
@@ -467,13 +523,13 @@ struct SetupOut {
   int lanes_a, lanes_t, lanes_ka, lanes_kt, th_a, th_t, nlong_a, nlong_t;
   int tiles, n_ta, n_tt;  // staged tile kernels built; their items over A and A^T
   int res_G;              // blocks of the resident step kernel (0: not planned)
-  void* res_base;         // its buffers
+  ResBufs rb;             // its buffers
   ResSizes res;
 };
 
-// The form of the step attempts of one LP with float32 iterates where the caller asks for none
-// (persistent = 0 without lanes, tiles, the autotuner or the Halpern variant): the LP in one
-// block's shared memory up to kOneBlockNnz nonzeros, spread over the SMs' shared memory
+// The form of the step attempts of one LP where the caller asks for none (persistent = 0 without
+// lanes, tiles, the autotuner or the Halpern variant): with float32 iterates the LP in one block's
+// shared memory up to kOneBlockNnz nonzeros; spread over the SMs' shared memory
 // (resident_kernels.cuh) while it fits there, else three launches per attempt.  Measured per
 // attempt on a GB300 (us; values in float32 / bfloat16 or the 0/1 pattern):
 //                                 nonzeros   three launches   one block     resident
@@ -485,35 +541,34 @@ struct SetupOut {
 //   covering 50,000 x 200,000    1,350,409     23.0 / 20.5                 20.3 / 13.7
 //   energy system, 24 h             21,600     23.3                         4.9
 //   energy system, 720 h           648,000     17.7                        10.4
-// kResNnz nonzeros per block: 256 and 1,024 measured within 10 % of 512, slower on most.
-constexpr int kResNnz = 512;
+// and in float64 (one block would win nothing: its chains of float64 operations are as long):
+//   relaxation 40 x 80                 320     15.5             6.4           5.6
+//   relaxation 200 x 400             1,670     16.6             7.7           7.9
+//   relaxation 2,000 x 4,000        15,963     19.1                           8.7
+//   covering 2,000 x 8,000          54,130     25.8                          10.4
+//   covering 10,000 x 40,000       269,989     33.7                          14.4
+//   covering 25,000 x 100,000      675,211     40.0                          27.7
+//   energy system, 24 h             21,600     23.7                          10.8
+//   energy system, 400 h           360,000    129.0                          18.5
+// kResNnz nonzeros per block: 256 and 1,024 measured within 10 % of 512, slower on most; in
+// float64 256 (128: 3-6 % slower, 512: 2 % faster to 10 % slower).
+constexpr int kResNnz = 512, kResNnz64 = 256;
 constexpr int kOneBlockNnz = 2500;
-static bool auto_form(const pdlp_params* p, Mode mode, int m, long long nnz) {
-  return mode != MODE_FP64 && p->persistent == 0 && !p->tiles && !p->halpern && !p->autotune &&
-         !p->lanes_A && !p->lanes_AT && m > 0 && nnz > 0;
+static int one_block_nnz(Mode mode) { return mode == MODE_FP64 ? 0 : kOneBlockNnz; }
+// Float64 solves that record iterates or decisions are parity runs against a reference: they keep
+// the separate launches, whose order of summation such records were made with.
+static bool parity_run(Mode mode, const pdlp_diagnostics* dg) {
+  return mode == MODE_FP64 && dg &&
+         (dg->x_cur || dg->y_cur || dg->x_avg || dg->y_avg || dg->attempt_capacity > 0);
 }
-static int resident_blocks(long long nnz) {
-  return (int)std::max(1LL, std::min<long long>(device_sm_count(), nnz / kResNnz));
+static bool auto_form(const pdlp_params* p, int m, long long nnz) {
+  return p->persistent == 0 && !p->tiles && !p->halpern && !p->autotune && !p->lanes_A &&
+         !p->lanes_AT && m > 0 && nnz > 0;
 }
-// Buffers of the resident step kernel, from `base` on (256-byte aligned).
-struct ResBufs {
-  ulonglong2 *slot, *ex_x;
-  unsigned long long* ex_y;  // [2][m]
-  int *cut_t, *cut_a;
-  ResSizes* sizes;
-  size_t clear, bytes;  // the first `clear` bytes start as zeros (no tag)
-  ResBufs(void* base, int G, long long m, long long n) {
-    Arena ar{(char*)base, 0};
-    slot = (ulonglong2*)ar.take(16 * (size_t)kResReplicas * G);
-    ex_x = (ulonglong2*)ar.take(16 * (size_t)n);
-    ex_y = (unsigned long long*)ar.take(8 * 2 * (size_t)m);
-    clear = ar.off;
-    cut_t = (int*)ar.take(4 * ((size_t)G + 1));
-    cut_a = (int*)ar.take(4 * ((size_t)G + 1));
-    sizes = (ResSizes*)ar.take(sizeof(ResSizes));
-    bytes = ar.off;
-  }
-};
+static int resident_blocks(Mode mode, long long nnz) {
+  const long long per = mode == MODE_FP64 ? kResNnz64 : kResNnz;
+  return (int)std::max(1LL, std::min<long long>(device_sm_count(), nnz / per));
+}
 static int optin_smem() {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
@@ -531,7 +586,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
                     const int* forced_lanes, SetupOut* so, const double* hx = nullptr,
                     const double* hy = nullptr,
                     const std::function<void(const char*)>& mark = [](const char*) {},
-                    bool build_tiles = true) {
+                    bool build_tiles = true, const pdlp_diagnostics* dg = nullptr) {
   const int m = A->m, n = A->n;
   const long long nnz = A->nnz;
   // ---- validation (A0 preconditions)
@@ -628,23 +683,33 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
     g_launches += 10;
   }
   // the parts of the resident step kernel, if the LP's data can fit on the chip at all and its
-  // buffers in scratch that is free by now: the scalars' partial sums or the transpose's
+  // buffers in scratch that is free by now: the scalars' partial sums or the transpose's, and in
+  // float64, where they are twice as large, those and the scaling's statistics and the step
+  // weights of the other storage form
   so->res_G = 0;
-  so->res_base = nullptr;
+  so->rb = ResBufs{};
   so->res = ResSizes{};
-  if (auto_form(p, mode, m, nnz) && nnz > kOneBlockNnz) {
-    const int vb = mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
-    const long long data = nnz * 2 * (4 + vb) + 24LL * ((long long)m + n);
-    const int G = resident_blocks(nnz);
-    const size_t need = ResBufs(nullptr, G, m, n).bytes;
-    so->res_base = need <= 8 * setup_part_doubles(m, n) ? (void*)bf.part_setup
-                   : need <= bf.tmp_bytes               ? (void*)bf.tmp
-                                                        : nullptr;
-    if (so->res_base && data <= (long long)device_sm_count() * optin_smem()) {
+  if (auto_form(p, m, nnz) && nnz > one_block_nnz(mode) && !parity_run(mode, dg)) {
+    const int it = mode == MODE_FP64 ? 8 : 4;
+    const int vb = mode == MODE_FP64 ? 8 : mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
+    const long long data = nnz * 2 * (4 + vb) + 6LL * it * ((long long)m + n);
+    const int G = resident_blocks(mode, nnz);
+    const Region part{bf.part_setup, 8 * setup_part_doubles(m, n)}, tmp{bf.tmp, bf.tmp_bytes};
+    if (mode == MODE_FP64) {
+      auto upto = [](void* from, void* last, size_t bytes) {  // neighbours in the workspace
+        return Region{from, (size_t)((char*)last + bytes - (char*)from)};
+      };
+      const Region all[4] = {part, upto(bf.stat_r, bf.stat_c, 8 * (size_t)n),
+                             upto(bf.tw, bf.sw, 8 * (size_t)m), tmp};
+      so->rb.place(all, 4, G, m, n, it);
+    } else if (!so->rb.place(&part, 1, G, m, n, it)) {
+      so->rb.place(&tmp, 1, G, m, n, it);
+    }
+    const ResBufs& rb = so->rb;
+    if (rb.ok && data <= (long long)device_sm_count() * optin_smem()) {
       so->res_G = G;
-      const ResBufs rb(so->res_base, G, m, n);
-      CUDA_TRY(setup_res_plan(m, n, (int)nnz, bf.a_ptr, bf.t_ptr, G, vb, mode != MODE_FP32,
-                              rb.cut_t, rb.cut_a, rb.sizes, s));
+      CUDA_TRY(setup_res_plan(m, n, (int)nnz, bf.a_ptr, bf.t_ptr, G, it, vb,
+                              mode == MODE_BF16 || mode == MODE_PAT, rb.cut_t, rb.cut_a, rb.sizes, s));
       CUDA_TRY(cudaMemcpyAsync(&so->res, rb.sizes, sizeof(ResSizes), cudaMemcpyDeviceToHost, s));
       ++g_launches;
     }
@@ -946,7 +1011,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
   SetupOut so;
   {
     const int rc = setup_lp(A, b, sense, c, l, u, p, x0, y0, bf, s, no_alloc, -1, nullptr, &so, hx,
-                            hy, phase);
+                            hy, phase, true, dg);
     if (rc) return rc;
   }
   phase("long rows + scalars");
@@ -1177,16 +1242,17 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
   }
   if (so.res_G > 0) {
     // an LP that fits in the SMs' shared memory
-    const ResBufs rb(so.res_base, so.res_G, m, n);
+    const ResBufs& rb = so.rb;
     const ResSizes& z = so.res;
+    const int it = mode == MODE_FP64 ? 8 : 4;
     ResPlan R{};
     R.G = so.res_G;
     R.cut_t = rb.cut_t;
     R.cut_a = rb.cut_a;
     R.slot = rb.slot;
     R.ex_x = rb.ex_x;
-    R.ex_y[0] = rb.ex_y;
-    R.ex_y[1] = rb.ex_y + m;
+    R.ex_y[0] = rb.ex_y[0];
+    R.ex_y[1] = rb.ex_y[1];
     auto bits = [](long long count) {  // bits of an index below count
       int k = 1;
       while ((1LL << k) < count) ++k;
@@ -1198,22 +1264,25 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     R.shift_a = std::max(0, R.bits_a - bits(kResBuckets));
     const int part = std::max(z.t_nnz, z.a_nnz);
     R.threads = part <= 1024 ? 256 : kResBlock;
-    auto lanes = [&](int rows) {  // as many lanes per row as one round of the block allows
+    // as many lanes per row as one round of the block allows (float64: with at most four
+    // entries of an average row each where fewer do that, since its pipe is what a shuffle
+    // level's additions hold)
+    auto lanes = [&](int rows, double avg) {
       int L = 1;
-      while (L < 16 && 2LL * L * rows <= R.threads) L <<= 1;
+      while (L < 16 && 2LL * L * rows <= R.threads && !(it == 8 && 4.0 * L >= avg)) L <<= 1;
       return L;
     };
-    R.lanes_t = lanes(z.t_rows);
-    R.lanes_a = lanes(z.a_rows);
+    R.lanes_t = lanes(z.t_rows, (double)nnz / n);
+    R.lanes_a = lanes(z.a_rows, (double)nnz / m);
     // the stage: a side's whole part where it fits, else as much as does (whole rows)
     const long long room = optin_smem() - kSmemStatic - (long long)z.bytes;
     const long long want =
-        (std::max({4LL * z.t_nnz, 8LL * z.a_nnz, 4LL * kResBuckets}) + 15) / 16 * 16;
+        (std::max({(long long)it * z.t_nnz, 2LL * it * z.a_nnz, 4LL * kResBuckets}) + 15) / 16 * 16;
     const long long stage = std::min(want, room / 16 * 16);
-    R.cap_t = (int)(stage / 4);
-    R.cap_a = (int)(stage / 8);
+    R.cap_t = (int)(stage / it);
+    R.cap_a = (int)(stage / (2 * it));
     R.smem = (int)(z.bytes + stage);
-    const bool fits = stage == want || stage >= 8LL * std::max(z.max_len, kResMinStage);
+    const bool fits = stage == want || stage >= 2LL * it * std::max(z.max_len, kResMinStage);
     if (fits && R.bits_t + bits(z.t_nnz) <= 32 && R.bits_a + bits(z.a_nnz) <= 32) {
       sv.ir.res = R;
       sv.persist_grid = R.G;
@@ -1221,13 +1290,14 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
         sv.ir.res = ResPlan{};
         sv.persist_grid = 0;
       } else {
-        CUDA_TRY(cudaMemsetAsync(rb.slot, 0, rb.clear, s));
+        CUDA_TRY(rb.clear(s));
       }
     }
   }
   // one block: asked for, or a small LP whose form is ours to choose (and which fits: below)
-  const bool small = auto_form(p, mode, m, nnz) && nnz <= kOneBlockNnz &&
-                     smem_layout(m, n, nnz, 4, mode != MODE_PAT, mode != MODE_FP32).bytes <=
+  const bool small = auto_form(p, m, nnz) && nnz <= one_block_nnz(mode) &&
+                     smem_layout(m, n, nnz, mode == MODE_FP64 ? 8 : 4, mode != MODE_PAT,
+                                 mode == MODE_BF16 || mode == MODE_PAT).bytes <=
                          optin_smem() - kSmemStatic;
   if (p->persistent || small) {
     // the resident grid of the persistent kernel (probe launch with nothing to do:
@@ -1276,7 +1346,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     CUDA_TRY(cudaStreamSynchronize(s));
     h1 = std::chrono::steady_clock::now();
   }
-  if (tq && !no_alloc) return time_kernels_after_setup(sv, bf.st, mode, nnz, *tq, 1);
+  if (tq && !no_alloc) return time_kernels_after_setup(sv, bf.st, mode, nnz, *tq, 1, &so.rb);
   if (no_alloc) {
     // the same chunk of step attempts and KKT block, launched directly on the
     // caller's stream; the four-byte status is read into pageable memory
@@ -1526,7 +1596,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
 }
 
 static int time_kernels_after_setup(Solve& sv, DevState* st, int mode, long long nnz,
-                                    const TimingReq& tq, int count) {
+                                    const TimingReq& tq, int count, const ResBufs* rb) {
   const cudaStream_t s = sv.s;
   const int m = sv.m, n = sv.n;
   // the state every timing starts from (one per LP of a batch): every step attempt stays
@@ -1568,8 +1638,8 @@ static int time_kernels_after_setup(Solve& sv, DevState* st, int mode, long long
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     cudaError_t ce = cudaSuccess;
     // reps attempts inside one launch (posted words of an earlier run would carry its tags)
-    if (which == 5 && sv.ir.res.G > 0)
-      ce = cudaMemsetAsync(sv.ir.res.slot, 0, ResBufs(sv.ir.res.slot, sv.ir.res.G, m, n).clear, cs);
+    if (which == 5 && rb && sv.ir.res.G > 0)
+      ce = rb->clear(cs);
     if (which == 5 && ce == cudaSuccess) ce = cap.persist(tq.reps);
     for (int i = 0; i < tq.reps && ce == cudaSuccess && which != 5; ++i) {
       if (which == 0 || which == 2) ce = cap.iter(IK_PRIMAL);

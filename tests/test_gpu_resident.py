@@ -1,8 +1,9 @@
-"""The resident step kernel (persistent_form 4: one LP with float32 iterates spread over the SMs'
-shared memory) and the rule that chooses it.
+"""The resident step kernel (persistent_form 4: one LP spread over the SMs' shared memory) and the
+rule that chooses it.
 
 Iterates after 60 fixed steps agree with the float64 oracle's and with the separate launches' to
-float32 rounding (a few hundred roundings of 6e-8: 2e-5, as for the other forms).  The sizes put
+rounding (a few hundred roundings: of 6e-8 in float32, 2e-5 as for the other forms; of 1.1e-16 in
+float64, 1e-12).  The sizes put
 rows and columns at the lengths where a warp takes over (64, 65), parts into several stages, and
 blocks without rows.
 """
@@ -16,7 +17,7 @@ from oracle import pdlp_oracle as O
 
 pytestmark = pytest.mark.gpu
 
-F32 = 2e-5
+F32, F64 = 2e-5, 1e-12
 FIXED = dict(adaptive_step=0, restarts=0, terminate=0, fixed_eta=0.9, iter_limit=60)
 
 
@@ -59,6 +60,7 @@ LPS = {
 # vectors that do not fit in the scratch the setup leaves (the workspace does not grow for them):
 # the separate launches run
 NOT_RESIDENT = {"empty_rows_and_columns"}
+NOT_RESIDENT_F64 = NOT_RESIDENT | {"one_long_row", "some_empty_rows_and_columns"}  # (twice the size)
 
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
@@ -78,6 +80,21 @@ def test_resident_iterates(P, name, prec):
         assert rel(it[k], getattr(ref, k)) <= F32, (k, rel(it[k], getattr(ref, k)))
 
 
+@pytest.mark.parametrize("name", list(LPS))
+def test_resident_float64(P, name):
+    """(A solve that records iterates keeps the separate launches: the points are compared.)"""
+    lp = LPS[name]()
+    x, y, r = P.pdlp_solve(lp, P.default_params(**FIXED))
+    x0, y0, r0 = P.pdlp_solve(lp, P.default_params(lanes_A=2, lanes_AT=2, **FIXED))
+    assert r["persistent_form"] == (0 if name in NOT_RESIDENT_F64 else 4)
+    assert r0["persistent_form"] == 0
+    assert P.pdlp_solve(lp, P.default_params(**FIXED), iterates=True)[2]["persistent_form"] == 0
+    ref = O.solve(lp, O.Params(iter_limit=60, adaptive=False, restarts=False, terminate=False,
+                               fixed_eta=0.9))
+    for got, want in ((x, x0), (y, y0), (x, ref.x), (y, ref.y)):
+        assert rel(got, want) <= F64, rel(got, want)
+
+
 def test_several_stages(P):
     """The 50,000 x 200,000 covering LP with float32 values: the entries of a part are staged
     in more than one go."""
@@ -89,6 +106,17 @@ def test_several_stages(P):
     assert r["persistent_form"] == 4
     for k in ("x_cur", "y_cur", "x_avg", "y_avg"):
         assert rel(it[k], it0[k]) <= F32, (k, rel(it[k], it0[k]))
+
+
+def test_rejected_steps_float64(P):
+    """As below; a rounding grows about tenfold every 40 adaptive steps, 1e-9 after 100."""
+    lp = lpgen.set_cover(5, m=1500, n=6000)
+    prm = dict(fixed_eta=200.0, iter_limit=100, terminate=0)
+    x, y, r = P.pdlp_solve(lp, P.default_params(**prm))
+    x0, y0, r0 = P.pdlp_solve(lp, P.default_params(lanes_A=2, lanes_AT=2, **prm))
+    assert r["persistent_form"] == 4 and r0["persistent_form"] == 0
+    assert r["attempts"] == r0["attempts"] > r["iters"] == 100
+    assert rel(x, x0) <= 1e-9 and rel(y, y0) <= 1e-9
 
 
 def test_rejected_steps(P):
@@ -109,7 +137,9 @@ def test_form_by_size(P):
 
     small, mid = lpgen.mip_relaxation(1), lpgen.set_cover(7, m=2000, n=8000)
     assert form(small, precision="fp32") == 3 and form(mid, precision="fp32") == 4
-    for kw in (dict(precision="fp64"), dict(precision="fp32", lanes_A=2), dict(precision="bf16", autotune=1),
+    assert form(small, precision="fp64") == form(mid, precision="fp64") == 4
+    assert form(lpgen.set_cover(2025), precision="fp64") == 0  # more than the SMs hold
+    for kw in (dict(precision="fp64", lanes_A=2), dict(precision="fp32", lanes_A=2), dict(precision="bf16", autotune=1),
                dict(precision="fp32", tiles=1), dict(precision="fp32", halpern=1)):
         assert form(small, **kw) == form(mid, **kw) == 0, kw
     assert form(lpgen.energy_system(hours=2880), precision="fp32") == 0  # more than the SMs hold
