@@ -7,9 +7,9 @@
 //   k_gnn_spmm                                       message passing over A or A^T (16 lanes
 //                                                    per row, one float4 of the 64-wide
 //                                                    hidden row per lane)
-//   k_gnn_dense / k_gnn_dense_bwd                    relu(X1 W1 + X2 W2 + b) on 64-row tiles
-//                                                    staged in shared memory, and its
-//                                                    backward (input and weight gradients)
+//   k_gnn_dense / k_gnn_dense_bwd                    relu(X1 W1 + X2 W2 + b) on the tensor cores,
+//                                                    16 rows per warp, and its backward (input
+//                                                    and weight gradients, 64 rows per block)
 //   k_gnn_head                                       prediction heads, loss and their gradient
 //   k_gnn_reduce / k_gnn_loss                        per-block partials summed in a fixed
 //                                                    order (training is deterministic)
@@ -40,8 +40,6 @@ namespace {
 using bf16 = __nv_bfloat16;
 constexpr int H = GNN_HIDDEN;
 constexpr int NB = 256;  // threads per block of every kernel here
-constexpr int kDenseSmem = (128 * 64 + 64 * 132) * 4;
-constexpr int kBwdSmem = (2 * 64 * 64 + 3 * 64 * 68) * 4;
 constexpr int kDensePart = 2 * 4096 + 64;
 
 int gfail(int code, const std::string& msg) {
@@ -119,6 +117,8 @@ int grid_rows(long long rows, int rows_per_block, int cap) {
   return (int)std::max<long long>(1, std::min<long long>(g, cap));
 }
 
+constexpr int kAnyGrid = 0x7fffffff;  // one round of rows per block, however many blocks
+
 // ---------------------------------------------------------------- device helpers
 __device__ __forceinline__ float bf(bf16 v) { return __bfloat162float(v); }
 
@@ -176,6 +176,14 @@ __global__ void k_gnn_stats(int rows, const int* __restrict__ ptr, const double*
     atomicMax(&maxes[0], m0);
     atomicMax(&maxes[1], m1);
     atomicMax(&maxes[2], m2);
+  }
+}
+
+__global__ void k_gnn_values(int nnz, const double* __restrict__ a, const double* __restrict__ t,
+                             float* __restrict__ a32, float* __restrict__ t32) {
+  for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += gridDim.x * blockDim.x) {
+    a32[i] = (float)a[i];
+    t32[i] = (float)t[i];
   }
 }
 
@@ -250,6 +258,7 @@ __global__ void __launch_bounds__(NB) k_gnn_embed_bwd(int N, const float* __rest
   float g[NF + 1];
 #pragma unroll
   for (int f = 0; f <= NF; ++f) g[f] = 0.f;
+#pragma unroll 4  // rows in flight
   for (long long r = (long long)blockIdx.x * 4 + rl; r < N; r += (long long)gridDim.x * 4) {
     const float d = H0[r * H + h] > 0.f ? dH0[r * H + h] : 0.f;
 #pragma unroll
@@ -265,9 +274,14 @@ __global__ void __launch_bounds__(NB) k_gnn_embed_bwd(int N, const float* __rest
 
 // ---------------------------------------------------------------- message passing (K12)
 // out[r] (+)= srow[r] * sum_k val[k] * scol[col[k]] * X[col[k]]  (srow / scol may be NULL = 1)
-__global__ void __launch_bounds__(NB) k_gnn_spmm(int rows, const int* __restrict__ ptr,
+// What is left is the gathers (173 MB from L2 for the 650,000 entries of a 25,000 x 100,000
+// covering LP).  The graph keeps the values in float32: converted here by every lane they held the
+// float64 pipe for half of the time.  Both directions of that LP: 26.5 -> 14.5 and 30.8 -> 16.5 us;
+// handing entries round by shuffles instead (one conversion each) 19.6 and 24.7; a warp per row, or
+// eight gathers in flight per lane, is no faster.
+__global__ void __launch_bounds__(NB, 6) k_gnn_spmm(int rows, const int* __restrict__ ptr,
                                                  const int* __restrict__ col,
-                                                 const double* __restrict__ val,
+                                                 const float* __restrict__ val,
                                                  const float* __restrict__ srow,
                                                  const float* __restrict__ scol,
                                                  const float* __restrict__ X, float* __restrict__ out,
@@ -285,7 +299,7 @@ __global__ void __launch_bounds__(NB) k_gnn_spmm(int rows, const int* __restrict
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         j[t] = col[k + t];
-        w[t] = (float)val[k + t];
+        w[t] = val[k + t];
       }
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
@@ -302,7 +316,7 @@ __global__ void __launch_bounds__(NB) k_gnn_spmm(int rows, const int* __restrict
     }
     for (; k < k1; ++k) {
       const int jj = col[k];
-      float w = (float)val[k];
+      float w = val[k];
       if (scol) w *= scol[jj];
       const float4 x = ld4(X + (size_t)jj * H + 4 * q);
       acc.x = fmaf(w, x.x, acc.x);
@@ -330,196 +344,319 @@ __global__ void __launch_bounds__(NB) k_gnn_spmm(int rows, const int* __restrict
 }
 
 // ---------------------------------------------------------------- dense layers (K13)
+// The layers' products run on the tensor cores from exact pieces: a float32 operand is the sum of
+// three bfloat16 numbers (its top 8 significant bits, the next 8 and the last 8, by truncation:
+// Ozaki et al., "Error-free transformations of matrix multiplication", 2012), the weights are
+// bfloat16, and a product of two bfloat16 numbers is exact in float32.  Every 16 terms of a sum
+// are multiplied and added by the matrix unit from zero and the 16-term sums added in float32
+// registers.  The unit cuts its sums off, a bias that a gradient adds up over all the rows; so the
+// sum d of the top pieces is followed by the same products less d, which gives what was cut off,
+// and the small pieces go on top of that (mma_add).
+// Measured with the LP of 100,000 columns (cold, ncu): a forward layer 62.8 us with float32
+// multiply-adds, 25 without the remainder (relative error of a gradient against float64 1.3e-7
+// instead of 5e-8: not kept), 34.5 as here (5.0e-8; the predictions' 3.8e-8 / 5.1e-8 before
+// 4.6e-8 / 5.6e-8); 50,000 columns backward 58.9 -> 45.3 us.  What bounds it is the issue of the
+// warp-level mma.sync (one in about 24 cycles per SM quarter at every mix tried).  tcgen05.mma is
+// not used: the remainder needs the accumulator in registers and negated after every 16 terms.
+using u32 = unsigned;
+
+// the pieces of (a, b), packed two to a word; an infinity is all in the first piece
+__device__ __forceinline__ void split_pair(float a, float b, u32& h, u32& m, u32& l) {
+  const u32 top = 0xffff0000u;
+  const float ha = __uint_as_float(__float_as_uint(a) & top), hb = __uint_as_float(__float_as_uint(b) & top);
+  const float ra = ha == a ? 0.f : a - ha, rb = hb == b ? 0.f : b - hb;
+  const float ma = __uint_as_float(__float_as_uint(ra) & top), mb = __uint_as_float(__float_as_uint(rb) & top);
+  const float la = ra - ma, lb = rb - mb;
+  h = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+  m = __byte_perm(__float_as_uint(ra), __float_as_uint(rb), 0x7632);
+  l = __byte_perm(__float_as_uint(la), __float_as_uint(lb), 0x7632);
+}
+
+// d += A B for a 16 x 16 A (row-major fragments) and a 16 x 8 B (column-major)
+__device__ __forceinline__ void mma16(float (&d)[4], const u32 (&a)[4], u32 b0, u32 b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// acc += d + r for d = the top pieces' products and r, begun from their remainder by `rest`, the
+// others' (an infinite or undefined d has no remainder)
+template <typename Rest>
+__device__ __forceinline__ void mma_add(float (&acc)[4], const u32 (&a)[4], u32 b0, u32 b1, Rest rest) {
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
+  mma16(d, a, b0, b1);
+  float r[4] = {-d[0], -d[1], -d[2], -d[3]};
+  mma16(r, a, b0, b1);
+  rest(r);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) acc[e] = (acc[e] + (fabsf(d[e]) < INFINITY ? r[e] : 0.f)) + d[e];
+}
+// four 8 x 8 matrices of 16-bit elements; lane 8j + i points at row i of matrix j
+__device__ __forceinline__ void ldsm4(u32 (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((u32)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(u32 (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((u32)__cvta_generic_to_shared(p))
+               : "memory");
+}
+
 // out = relu(X1 W1 + X2 W2 + b) for X1, X2 [N][64], W [64][64] row-major [in][out].
-// A block stages both weights (as float) once and then 64-row tiles of [X1 | X2];
-// thread (ty, tx) computes rows 4ty..4ty+3 x columns 4tx..4tx+3.
-__global__ void __launch_bounds__(NB) k_gnn_dense(int N, const float* __restrict__ X1,
-                                                  const float* __restrict__ X2,
-                                                  const bf16* __restrict__ W1,
-                                                  const bf16* __restrict__ W2,
-                                                  const bf16* __restrict__ bias,
-                                                  float* __restrict__ out) {
-  extern __shared__ float4 smem4[];
-  float* Ws = reinterpret_cast<float*>(smem4);  // [128][64]
-  float* Xs = Ws + 128 * 64;                    // [64][132]
-  for (int i = threadIdx.x; i < 64 * 64; i += NB) {
-    Ws[i] = bf(W1[i]);
-    Ws[64 * 64 + i] = bf(W2[i]);
+// A warp takes 16 rows at a time straight from global memory: lane (g, t) of a fragment holds
+// columns 4t..4t+3 of each 16-column chunk of rows g and g + 8 (one 16-byte load; the weights are
+// read in the same order of the sum), the 64 columns of the next step in flight meanwhile.
+constexpr int kDStride = 72;  // bf16 per row of weights in shared memory: an odd number of 16-byte
+                              // units, so that ldmatrix meets no bank twice
+__device__ __forceinline__ void stage_weights(bf16* Ws, const bf16* __restrict__ W1,
+                                              const bf16* __restrict__ W2) {
+  // (a layer's weights start at any even offset of the parameters: 4-byte loads)
+  for (int i = threadIdx.x; i < 64 * 32; i += NB) {
+    const int k = i >> 5, h = 2 * (i & 31);
+    *reinterpret_cast<u32*>(Ws + k * kDStride + h) = *reinterpret_cast<const u32*>(W1 + 2 * i);
+    *reinterpret_cast<u32*>(Ws + (64 + k) * kDStride + h) = *reinterpret_cast<const u32*>(W2 + 2 * i);
   }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float b4[4];
+}
+__global__ void __launch_bounds__(NB, 2) k_gnn_dense(int N, const float* __restrict__ X1,
+                                                     const float* __restrict__ X2,
+                                                     const bf16* __restrict__ W1,
+                                                     const bf16* __restrict__ W2,
+                                                     const bf16* __restrict__ bias,
+                                                     float* __restrict__ out) {
+  __shared__ __align__(16) bf16 Ws[128 * kDStride];  // [in of X1 | in of X2][out]
+  __shared__ __align__(8) float bs[64];
+  if (threadIdx.x < 64) bs[threadIdx.x] = bf(bias[threadIdx.x]);
+  stage_weights(Ws, W1, W2);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // the rows of the weights that a fragment's columns 4t..4t+3 of a chunk stand for: rows 2t, 2t+1
+  // of the first matrix are 4t, 4t+1, those of the second 4t+2, 4t+3
+  const int i8 = lane & 7, j4 = lane >> 3;
+  const bf16* wrow = Ws + (4 * (i8 >> 1) + (i8 & 1) + 2 * (j4 & 1)) * kDStride + 8 * (j4 >> 1);
+  const int tiles = (N + 15) / 16, step = gridDim.x * (NB / 32);
+  int w = blockIdx.x * (NB / 32) + (threadIdx.x >> 5), half = 0;
+  if (w >= tiles) return;
+  float4 nx[2][4];  // the four chunks of the next half (X1 or X2) of these or the next rows
+  auto load = [&](int tile, int hf) {
+    const float* X = hf ? X2 : X1;
+    const long long r0 = (long long)tile * 16 + g, r1 = r0 + 8;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) b4[e] = bf(bias[4 * tx + e]);
-  const int tiles = (N + 63) / 64;
-  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const long long row0 = (long long)t * 64;
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < 64 * 32; idx += NB) {
-      const int r = idx >> 5, qq = idx & 31;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row0 + r < N)
-        v = qq < 16 ? ld4(X1 + (row0 + r) * H + 4 * qq) : ld4(X2 + (row0 + r) * H + 4 * (qq - 16));
-      st4(Xs + r * 132 + 4 * qq, v);
+    for (int c = 0; c < 4; ++c) {
+      nx[0][c] = r0 < N ? ld4(X + r0 * H + 16 * c + 4 * t) : make_float4(0.f, 0.f, 0.f, 0.f);
+      nx[1][c] = r1 < N ? ld4(X + r1 * H + 16 * c + 4 * t) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
-    float acc[4][4];
+  };
+  load(w, 0);
+  float acc[8][4];
+#pragma unroll 1
+  while (w < tiles) {
+    float4 x[2][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int c = 0; c < 4; ++c) {
+      x[0][c] = nx[0][c];
+      x[1][c] = nx[1][c];
+    }
+    load(half ? w + step : w, half ^ 1);
+    if (half == 0)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = b4[j];
-#pragma unroll 4
-    for (int k4 = 0; k4 < 32; ++k4) {
-      float4 xr[4], w[4];
+      for (int j = 0; j < 8; ++j) {
+        const float2 b2 = *reinterpret_cast<const float2*>(bs + 8 * j + 2 * t);
+        acc[j][0] = acc[j][2] = b2.x;
+        acc[j][1] = acc[j][3] = b2.y;
+      }
+    const bf16* wt = wrow + 64 * half * kDStride;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) xr[i] = ld4(Xs + (4 * ty + i) * 132 + 4 * k4);
+    for (int c = 0; c < 4; ++c) {
+      u32 ah[4], am[4], al[4];
+      split_pair(x[0][c].x, x[0][c].y, ah[0], am[0], al[0]);
+      split_pair(x[1][c].x, x[1][c].y, ah[1], am[1], al[1]);
+      split_pair(x[0][c].z, x[0][c].w, ah[2], am[2], al[2]);
+      split_pair(x[1][c].z, x[1][c].w, ah[3], am[3], al[3]);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) w[kk] = ld4(Ws + (4 * k4 + kk) * 64 + 4 * tx);
+      for (int j = 0; j < 8; j += 2) {
+        u32 b[4];
+        ldsm4_t(b, wt + 16 * c * kDStride + 8 * j);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float xv[4] = {xr[i].x, xr[i].y, xr[i].z, xr[i].w};
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          acc[i][0] = fmaf(xv[kk], w[kk].x, acc[i][0]);
-          acc[i][1] = fmaf(xv[kk], w[kk].y, acc[i][1]);
-          acc[i][2] = fmaf(xv[kk], w[kk].z, acc[i][2]);
-          acc[i][3] = fmaf(xv[kk], w[kk].w, acc[i][3]);
+        for (int k = 0; k < 2; ++k) {
+          mma_add(acc[j + k], ah, b[2 * k], b[2 * k + 1], [&](float (&r)[4]) {
+            mma16(r, am, b[2 * k], b[2 * k + 1]);
+            mma16(r, al, b[2 * k], b[2 * k + 1]);
+          });
         }
       }
     }
+    if (half) {
+      const long long r0 = (long long)w * 16 + g, r1 = r0 + 8;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long r = row0 + 4 * ty + i;
-      if (r < N)
-        st4(out + r * H + 4 * tx, make_float4(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f),
-                                              fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f)));
+      for (int j = 0; j < 8; ++j) {
+        const int o = 8 * j + 2 * t;
+        if (r0 < N)
+          *reinterpret_cast<float2*>(out + r0 * H + o) = make_float2(fmaxf(acc[j][0], 0.f), fmaxf(acc[j][1], 0.f));
+        if (r1 < N)
+          *reinterpret_cast<float2*>(out + r1 * H + o) = make_float2(fmaxf(acc[j][2], 0.f), fmaxf(acc[j][3], 0.f));
+      }
+      w += step;
     }
+    half ^= 1;
   }
 }
 
 // Backward of k_gnn_dense: dP = dHn * (Hn > 0); dX1 = dP W1^T; dX2 = dP W2^T;
 // per-block partials of X1^T dP, X2^T dP (row-major [in][out]) and sum_r dP.
-__global__ void __launch_bounds__(NB) k_gnn_dense_bwd(int N, const float* __restrict__ X1,
-                                                      const float* __restrict__ X2,
-                                                      const float* __restrict__ Hn,
-                                                      const float* __restrict__ dHn,
-                                                      const bf16* __restrict__ W1,
-                                                      const bf16* __restrict__ W2,
-                                                      float* __restrict__ dX1,
-                                                      float* __restrict__ dX2,
-                                                      float* __restrict__ part) {
+// A block stages the pieces of 64 rows of [X1 | X2] and dP in shared memory; four warps form dX1
+// of the rows, four dX2 (16 rows each), then each warp its 16 of the 128 rows of the weight
+// gradients, where both operands are in pieces: the six products above 2^-24.
+// The rows of shared memory are padded to an odd number of 16-byte units (ldmatrix).
+constexpr int kXStride = 136, kBwdRows = 64;
+constexpr int kBwdSmem = (3 * kBwdRows * (kXStride + kDStride) + 128 * kDStride) * 2;
+__device__ __forceinline__ void split_store(bf16* p, int piece_stride, float4 v) {
+  uint2 h, m, l;
+  split_pair(v.x, v.y, h.x, m.x, l.x);
+  split_pair(v.z, v.w, h.y, m.y, l.y);
+  *reinterpret_cast<uint2*>(p) = h;
+  *reinterpret_cast<uint2*>(p + piece_stride) = m;
+  *reinterpret_cast<uint2*>(p + 2 * piece_stride) = l;
+}
+__global__ void __launch_bounds__(NB, 2) k_gnn_dense_bwd(int N, const float* __restrict__ X1,
+                                                         const float* __restrict__ X2,
+                                                         const float* __restrict__ Hn,
+                                                         const float* __restrict__ dHn,
+                                                         const bf16* __restrict__ W1,
+                                                         const bf16* __restrict__ W2,
+                                                         float* __restrict__ dX1,
+                                                         float* __restrict__ dX2,
+                                                         float* __restrict__ part) {
   extern __shared__ float4 smem4[];
-  float* Wt1 = reinterpret_cast<float*>(smem4);  // [64 out][64 in]
-  float* Wt2 = Wt1 + 64 * 64;
-  float* dPs = Wt2 + 64 * 64;                    // [64 rows][68]
-  float* X1s = dPs + 64 * 68;
-  float* X2s = X1s + 64 * 68;
-  for (int i = threadIdx.x; i < 64 * 64; i += NB) {
-    const int k = i >> 6, h = i & 63;  // W[k][h] -> Wt[h][k]
-    Wt1[h * 64 + k] = bf(W1[i]);
-    Wt2[h * 64 + k] = bf(W2[i]);
-  }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float g1[4][4], g2[4][4], gb = 0.f;
+  constexpr int XP = kBwdRows * kXStride, DP = kBwdRows * kDStride;
+  bf16* Xs = reinterpret_cast<bf16*>(smem4);  // [piece][row][in of X1 | in of X2]
+  bf16* Ds = Xs + 3 * XP;                     // [piece][row][out]
+  bf16* Ws = Ds + 3 * DP;                     // [in of W1 | in of W2][out]
+  stage_weights(Ws, W1, W2);
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int q = threadIdx.x & 15, rs = threadIdx.x >> 4;
+  const int i8 = lane & 7, j4 = lane >> 3;  // ldmatrix: row i8 of matrix j4
+  float gw[8][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) g1[i][j] = g2[i][j] = 0.f;
-  const int tiles = (N + 63) / 64;
-  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const long long row0 = (long long)t * 64;
+    for (int e = 0; e < 4; ++e) gw[j][e] = 0.f;
+  float4 gb = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int tiles = (N + kBwdRows - 1) / kBwdRows;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const long long row0 = (long long)tile * kBwdRows;
     __syncthreads();
-    for (int idx = threadIdx.x; idx < 64 * 16; idx += NB) {
-      const int r = idx >> 4, qq = idx & 15;
+#pragma unroll
+    for (int k = 0; k < kBwdRows / 16; ++k) {
+      const int r = rs + 16 * k;
       float4 d = make_float4(0.f, 0.f, 0.f, 0.f), a = d, b = d;
       if (row0 + r < N) {
-        const long long o = (row0 + r) * H + 4 * qq;
-        const float4 hn = ld4(Hn + o);
-        const float4 dh = ld4(dHn + o);
+        const long long o = (row0 + r) * H + 4 * q;
+        const float4 hn = ld4(Hn + o), dh = ld4(dHn + o);
         d = make_float4(hn.x > 0.f ? dh.x : 0.f, hn.y > 0.f ? dh.y : 0.f,
                         hn.z > 0.f ? dh.z : 0.f, hn.w > 0.f ? dh.w : 0.f);
         a = ld4(X1 + o);
         b = ld4(X2 + o);
       }
-      st4(dPs + r * 68 + 4 * qq, d);
-      st4(X1s + r * 68 + 4 * qq, a);
-      st4(X2s + r * 68 + 4 * qq, b);
+      gb.x += d.x;
+      gb.y += d.y;
+      gb.z += d.z;
+      gb.w += d.w;
+      split_store(Ds + r * kDStride + 4 * q, DP, d);
+      split_store(Xs + r * kXStride + 4 * q, XP, a);
+      split_store(Xs + r * kXStride + 64 + 4 * q, XP, b);
     }
     __syncthreads();
-    // input gradients: rows 4ty.., input columns 4tx..
-    {
-      float a1[4][4], a2[4][4];
+    {  // input gradients
+      const int rt = 16 * (wp & 3), half = wp >> 2;
+      float acc[8][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int j = 0; j < 8; ++j)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) a1[i][j] = a2[i][j] = 0.f;
-#pragma unroll 2
-      for (int h4 = 0; h4 < 16; ++h4) {
-        float4 d[4];
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = ld4(dPs + (4 * ty + i) * 68 + 4 * h4);
+      for (int c = 0; c < 4; ++c) {
+        u32 a[3][4];
 #pragma unroll
-        for (int hh = 0; hh < 4; ++hh) {
-          const float4 w1 = ld4(Wt1 + (4 * h4 + hh) * 64 + 4 * tx);
-          const float4 w2 = ld4(Wt2 + (4 * h4 + hh) * 64 + 4 * tx);
+        for (int p = 0; p < 3; ++p)
+          ldsm4(a[p], Ds + p * DP + (rt + (j4 & 1) * 8 + i8) * kDStride + 16 * c + (j4 >> 1) * 8);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float dv = hh == 0 ? d[i].x : (hh == 1 ? d[i].y : (hh == 2 ? d[i].z : d[i].w));
-            a1[i][0] = fmaf(dv, w1.x, a1[i][0]);
-            a1[i][1] = fmaf(dv, w1.y, a1[i][1]);
-            a1[i][2] = fmaf(dv, w1.z, a1[i][2]);
-            a1[i][3] = fmaf(dv, w1.w, a1[i][3]);
-            a2[i][0] = fmaf(dv, w2.x, a2[i][0]);
-            a2[i][1] = fmaf(dv, w2.y, a2[i][1]);
-            a2[i][2] = fmaf(dv, w2.z, a2[i][2]);
-            a2[i][3] = fmaf(dv, w2.w, a2[i][3]);
+        for (int j = 0; j < 8; j += 2) {
+          u32 b[4];
+          ldsm4(b, Ws + (64 * half + 8 * j + (j4 >> 1) * 8 + i8) * kDStride + 16 * c + (j4 & 1) * 8);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            mma_add(acc[j + k], a[0], b[2 * k], b[2 * k + 1], [&](float (&r)[4]) {
+              mma16(r, a[1], b[2 * k], b[2 * k + 1]);
+              mma16(r, a[2], b[2 * k], b[2 * k + 1]);
+            });
           }
         }
       }
+      float* dX = half ? dX2 : dX1;
+      const long long r0 = row0 + rt + g, r1 = r0 + 8;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const long long r = row0 + 4 * ty + i;
-        if (r < N) {
-          st4(dX1 + r * H + 4 * tx, make_float4(a1[i][0], a1[i][1], a1[i][2], a1[i][3]));
-          st4(dX2 + r * H + 4 * tx, make_float4(a2[i][0], a2[i][1], a2[i][2], a2[i][3]));
+      for (int j = 0; j < 8; ++j) {
+        const int o = 8 * j + 2 * t;
+        if (r0 < N) *reinterpret_cast<float2*>(dX + r0 * H + o) = make_float2(acc[j][0], acc[j][1]);
+        if (r1 < N) *reinterpret_cast<float2*>(dX + r1 * H + o) = make_float2(acc[j][2], acc[j][3]);
+      }
+    }
+    // weight gradients: inputs 16 wp .. of [X1 | X2], the sum over the rows
+#pragma unroll
+    for (int c = 0; c < kBwdRows / 16; ++c) {
+      u32 a[3][4];
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        ldsm4_t(a[p], Xs + p * XP + (16 * c + (j4 >> 1) * 8 + i8) * kXStride + 16 * wp + (j4 & 1) * 8);
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        u32 b[3][4];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          ldsm4_t(b[p], Ds + p * DP + (16 * c + (j4 & 1) * 8 + i8) * kDStride + 8 * j + (j4 >> 1) * 8);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          mma_add(gw[j + k], a[0], b[0][2 * k], b[0][2 * k + 1], [&](float (&r)[4]) {
+            mma16(r, a[1], b[0][2 * k], b[0][2 * k + 1]);
+            mma16(r, a[0], b[1][2 * k], b[1][2 * k + 1]);
+            mma16(r, a[1], b[1][2 * k], b[1][2 * k + 1]);
+            mma16(r, a[2], b[0][2 * k], b[0][2 * k + 1]);
+            mma16(r, a[0], b[2][2 * k], b[2][2 * k + 1]);
+          });
         }
       }
     }
-    // weight gradients: inputs 4ty.., outputs 4tx..
-#pragma unroll 4
-    for (int r = 0; r < 64; ++r) {
-      const float4 x1 = ld4(X1s + r * 68 + 4 * ty);
-      const float4 x2 = ld4(X2s + r * 68 + 4 * ty);
-      const float4 d = ld4(dPs + r * 68 + 4 * tx);
-      const float xa[4] = {x1.x, x1.y, x1.z, x1.w}, xb[4] = {x2.x, x2.y, x2.z, x2.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        g1[i][0] = fmaf(xa[i], d.x, g1[i][0]);
-        g1[i][1] = fmaf(xa[i], d.y, g1[i][1]);
-        g1[i][2] = fmaf(xa[i], d.z, g1[i][2]);
-        g1[i][3] = fmaf(xa[i], d.w, g1[i][3]);
-        g2[i][0] = fmaf(xb[i], d.x, g2[i][0]);
-        g2[i][1] = fmaf(xb[i], d.y, g2[i][1]);
-        g2[i][2] = fmaf(xb[i], d.z, g2[i][2]);
-        g2[i][3] = fmaf(xb[i], d.w, g2[i][3]);
-      }
-    }
-    if (threadIdx.x < 64)
-      for (int r = 0; r < 64; ++r) gb += dPs[r * 68 + threadIdx.x];
   }
   float* p = part + (size_t)blockIdx.x * kDensePart;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    st4(p + (4 * ty + i) * 64 + 4 * tx, make_float4(g1[i][0], g1[i][1], g1[i][2], g1[i][3]));
-    st4(p + 4096 + (4 * ty + i) * 64 + 4 * tx, make_float4(g2[i][0], g2[i][1], g2[i][2], g2[i][3]));
+  for (int j = 0; j < 8; ++j) {
+    const int o = 8 * j + 2 * t, r = 16 * wp + g;
+    *reinterpret_cast<float2*>(p + r * 64 + o) = make_float2(gw[j][0], gw[j][1]);
+    *reinterpret_cast<float2*>(p + (r + 8) * 64 + o) = make_float2(gw[j][2], gw[j][3]);
   }
-  if (threadIdx.x < 64) p[8192 + threadIdx.x] = gb;
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(smem4);  // [16][64]
+  st4(red + rs * 64 + 4 * q, gb);
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    float sum = 0.f;
+    for (int r = 0; r < 16; ++r) sum += red[r * 64 + threadIdx.x];
+    p[8192 + threadIdx.x] = sum;
+  }
 }
 
 // ---------------------------------------------------------------- heads and loss
-// One half-warp per row (lane q holds hidden units 4q..4q+3).  MODE 0: primal head
+// A half-warp takes eight rows at a time (lane q holds hidden units 4q..4q+3 of each): the
+// products are reduced so that lanes 2i and 2i + 1 end with row i's, and each finishes its row (two
+// rows a warp instruction kept the float64 pipe busy with the boxes: 23.8 us for a covering LP's
+// 100,000 columns, now 10.8).  MODE 0: primal head
 // (l + (u - l) sigmoid on finite boxes), MODE 1: dual head (softplus on inequality
 // rows).  pred: float64 prediction in the caller's convention (may be NULL); with a
 // label: loss terms, dz, dH = dz w (may be NULL) and partials [64 gw | gb].
+constexpr int kHeadRows = 8 * 16;  // rows of a block at a time
 template <int MODE>
 __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict__ Hn,
                                                  const bf16* __restrict__ w,
@@ -541,17 +678,28 @@ __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict_
   float4 gw = make_float4(0.f, 0.f, 0.f, 0.f);
   float gb = 0.f;
   double ls = 0.0;
-  for (long long r = (long long)blockIdx.x * 16 + hw; r < N; r += (long long)gridDim.x * 16) {
-    const float4 h = ld4(Hn + r * H + 4 * q);
-    float z = h.x * wv.x + h.y * wv.y + h.z * wv.z + h.w * wv.w;
-    z += __shfl_xor_sync(mask, z, 8, 16);
-    z += __shfl_xor_sync(mask, z, 4, 16);
-    z += __shfl_xor_sync(mask, z, 2, 16);
-    z += __shfl_xor_sync(mask, z, 1, 16);
-    z += b0;
-    float p, dpdz, rng = 1.f;
+  for (long long r0 = ((long long)blockIdx.x * 16 + hw) * 8; r0 < N; r0 += (long long)gridDim.x * kHeadRows) {
+    float4 h[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      h[i] = r0 + i < N ? ld4(Hn + (r0 + i) * H + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = h[i].x * wv.x + h[i].y * wv.y + h[i].z * wv.z + h[i].w * wv.w;
+#pragma unroll
+    for (int o = 8, keep = 4; o > 1; o >>= 1, keep >>= 1)
+#pragma unroll
+      for (int i = 0; i < keep; ++i) {
+        const bool up = (q & o) != 0;
+        const float send = up ? v[i] : v[i + keep];
+        v[i] = (up ? v[i + keep] : v[i]) + __shfl_xor_sync(mask, send, o, 16);
+      }
+    const float z = v[0] + __shfl_xor_sync(mask, v[0], 1, 16) + b0;
+    const long long r = r0 + (q >> 1);
+    const bool live = r < N, lead = live && (q & 1) == 0;
+    float p = 0.f, dpdz = 0.f, rng = 1.f;
     unsigned char kd = 0;
-    if (MODE == 0) {
+    if (live && MODE == 0) {
       const double lj = l[r], uj = u[r];
       if (isfinite(lj) && isfinite(uj)) {
         const float s = sigmoidf(z), width = (float)(uj - lj);
@@ -562,7 +710,7 @@ __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict_
         p = z;
         dpdz = 1.f;
       }
-    } else {
+    } else if (live) {
       kd = kind[r];
       if (kd == 1) {
         p = z;
@@ -572,23 +720,34 @@ __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict_
         dpdz = sigmoidf(z);
       }
     }
-    if (pred && q == 0)
+    if (pred && lead)
       pred[r] = MODE == 0 ? (double)p : (kd == 2 ? -cmax * (double)p : cmax * (double)p);
     if (label) {
-      const float e = (p - label[r]) / rng;
-      const float dz = two_over_n * e / rng * dpdz;
-      if (q == 0) {
+      const float e = live ? (p - label[r]) / rng : 0.f;
+      const float dz = live ? two_over_n * e / rng * dpdz : 0.f;
+      if (lead) {
         ls += (double)e * (double)e;
         gb += dz;
       }
-      gw.x = fmaf(dz, h.x, gw.x);
-      gw.y = fmaf(dz, h.y, gw.y);
-      gw.z = fmaf(dz, h.z, gw.z);
-      gw.w = fmaf(dz, h.w, gw.w);
-      if (dH) st4(dH + r * H + 4 * q, make_float4(dz * wv.x, dz * wv.y, dz * wv.z, dz * wv.w));
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float di = __shfl_sync(mask, dz, 2 * i, 16);
+        if (r0 + i >= N) continue;
+        gw.x = fmaf(di, h[i].x, gw.x);
+        gw.y = fmaf(di, h[i].y, gw.y);
+        gw.z = fmaf(di, h[i].z, gw.z);
+        gw.w = fmaf(di, h[i].w, gw.w);
+        if (dH)
+          st4(dH + (r0 + i) * H + 4 * q, make_float4(di * wv.x, di * wv.y, di * wv.z, di * wv.w));
+      }
     }
   }
   if (!part) return;
+#pragma unroll
+  for (int o = 8; o > 1; o >>= 1) {  // (the odd lanes hold none)
+    gb += __shfl_xor_sync(mask, gb, o, 16);
+    ls += __shfl_xor_sync(mask, ls, o, 16);
+  }
   red[hw][q] = gw;
   if (q == 0) {
     redb[hw] = gb;
@@ -619,14 +778,23 @@ __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict_
 struct Seg {
   int src, len, dst;
 };
-// grad[dst + e] += scale * sum_b part[b * stride + src + e] in float64.  A block takes 32
-// elements: eight warps each add every eighth partial of them (one 128-byte line per warp and
-// partial), then one warp adds the eight sums in order.  One thread per element walked all 304
-// partials of a dense layer alone, 92 us of latency; now 13 us.
-__global__ void __launch_bounds__(NB) k_gnn_reduce(const float* __restrict__ part, int nblk,
-                                                   int stride, Seg s0, Seg s1, Seg s2,
-                                                   float* __restrict__ grad, float scale) {
-  __shared__ double sh[NB / 32][32];
+// a += x with the rounding error kept in e (Knuth's two-sum): float32 additions that together carry
+// twice the digits
+__device__ __forceinline__ void two_sum(float& a, float& e, float x) {
+  const float s = a + x, b = s - a;
+  e += (a - (s - b)) + (x - b);
+  a = s;
+}
+// grad[dst + e] += scale * sum_b part[b * stride + src + e].  A block takes 32 elements: 32 warps
+// each add every 32nd partial of them (one 128-byte line per warp and partial), then one warp adds
+// the 32 sums in order.  The sums are pairs of float32 numbers (an error of 2^-46, as good as the
+// float64 sums that they replace, whose conversions and additions held the float64 pipe: 2.5
+// million of each for the 304 partials of a dense layer; 15.0 -> 8.0 us on average).
+constexpr int kReduceNB = 1024;
+__global__ void __launch_bounds__(kReduceNB) k_gnn_reduce(const float* __restrict__ part, int nblk,
+                                                          int stride, Seg s0, Seg s1, Seg s2,
+                                                          float* __restrict__ grad, float scale) {
+  __shared__ float2 sh[kReduceNB / 32][32];
   const int total = s0.len + s1.len + s2.len, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
   Seg s = s0;
@@ -639,17 +807,21 @@ __global__ void __launch_bounds__(NB) k_gnn_reduce(const float* __restrict__ par
       s = s2;
     }
   }
-  double acc = 0.0;
+  float acc = 0.f, err = 0.f;
   if (e < total) {
     const float* p = part + s.src + i;
-#pragma unroll 8
-    for (int b = w; b < nblk; b += NB / 32) acc += (double)p[(size_t)b * stride];
+#pragma unroll 10
+    for (int b = w; b < nblk; b += kReduceNB / 32) two_sum(acc, err, p[(size_t)b * stride]);
   }
-  sh[w][lane] = acc;
+  sh[w][lane] = make_float2(acc, err);
   __syncthreads();
   if (w == 0 && e < total) {
-    for (int k = 1; k < NB / 32; ++k) acc += sh[k][lane];
-    grad[s.dst + i] += scale * (float)acc;
+    for (int k = 1; k < kReduceNB / 32; ++k) {
+      const float2 v = sh[k][lane];
+      two_sum(acc, err, v.x);
+      err += v.y;
+    }
+    grad[s.dst + i] += scale * (isfinite(acc) ? acc + err : acc);
   }
 }
 
@@ -1024,6 +1196,7 @@ struct gnn_graph {
   gnn_model* owner = nullptr;
   LpDev d;
   float *inv_deg_r = nullptr, *inv_deg_c = nullptr;
+  float *a_v32 = nullptr, *t_v32 = nullptr;  // the values of A and A^T as the layers use them
   float *fv = nullptr, *fc = nullptr;
   float *x_star = nullptr, *y_star = nullptr;  // labels: x*, y* (>=-form) / max|c|
   double cmax = 1.0;
@@ -1093,7 +1266,7 @@ int forward(gnn_model* md, gnn_graph* g, bool want_pred, bool with_label, bool w
   const int n = g->d.n, m = g->d.m;
   RTRY(ensure_scratch(md, n, m));
   cudaStream_t s = md->s;
-  const int Gs = sm_count() * 8, Gd = sm_count() * 3;
+  const int Gs = sm_count() * 8, Gd = sm_count() * 2;
   if (n > 0) {
     k_gnn_embed<GNN_VAR_FEATURES><<<grid_rows((long long)n, NB / 16, Gs), NB, 0, s>>>(
         n, g->fv, W(md, kOff.W_vin), W(md, kOff.b_vin), md->hv[0]);
@@ -1106,26 +1279,26 @@ int forward(gnn_model* md, gnn_graph* g, bool want_pred, bool with_label, bool w
   }
   for (int k = 0; k < GNN_LAYERS; ++k) {
     if (m > 0) {
-      k_gnn_spmm<<<grid_rows((long long)m, NB / 16, Gs), NB, 0, s>>>(
-          m, g->d.a_ptr, g->d.a_col, g->d.a_val, g->inv_deg_r, nullptr, md->hv[k], md->sc[k], 0);
+      k_gnn_spmm<<<grid_rows((long long)m, NB / 16, kAnyGrid), NB, 0, s>>>(
+          m, g->d.a_ptr, g->d.a_col, g->a_v32, g->inv_deg_r, nullptr, md->hv[k], md->sc[k], 0);
       GTRY(cudaGetLastError());
-      k_gnn_dense<<<grid_rows((long long)m, 64, Gd), NB, kDenseSmem, s>>>(
+      k_gnn_dense<<<grid_rows((long long)m, 128, Gd), NB, 0, s>>>(
           m, md->hc[k], md->sc[k], W(md, kOff.W_cc[k]), W(md, kOff.W_cv[k]), W(md, kOff.b_c[k]),
           md->hc[k + 1]);
       GTRY(cudaGetLastError());
     }
     if (n > 0) {
-      k_gnn_spmm<<<grid_rows((long long)n, NB / 16, Gs), NB, 0, s>>>(
-          n, g->d.t_ptr, g->d.t_col, g->d.t_val, g->inv_deg_c, nullptr, md->hc[k + 1], md->sv[k], 0);
+      k_gnn_spmm<<<grid_rows((long long)n, NB / 16, kAnyGrid), NB, 0, s>>>(
+          n, g->d.t_ptr, g->d.t_col, g->t_v32, g->inv_deg_c, nullptr, md->hc[k + 1], md->sv[k], 0);
       GTRY(cudaGetLastError());
-      k_gnn_dense<<<grid_rows((long long)n, 64, Gd), NB, kDenseSmem, s>>>(
+      k_gnn_dense<<<grid_rows((long long)n, 128, Gd), NB, 0, s>>>(
           n, md->hv[k], md->sv[k], W(md, kOff.W_vv[k]), W(md, kOff.W_vc[k]), W(md, kOff.b_v[k]),
           md->hv[k + 1]);
       GTRY(cudaGetLastError());
     }
   }
-  const int gx = grid_rows((long long)n, 16, md->max_blocks);
-  const int gy = grid_rows((long long)m, 16, md->max_blocks);
+  const int gx = grid_rows((long long)n, kHeadRows, md->max_blocks);
+  const int gy = grid_rows((long long)m, kHeadRows, md->max_blocks);
   if (n > 0) {
     k_gnn_head<0><<<gx, NB, 0, s>>>(n, md->hv[GNN_LAYERS], W(md, kOff.w_x), W(md, kOff.b_x),
                                     g->d.l, g->d.u, nullptr, g->cmax,
@@ -1154,7 +1327,7 @@ int forward(gnn_model* md, gnn_graph* g, bool want_pred, bool with_label, bool w
 
 int reduce_into(gnn_model* md, int nblk, int stride, Seg a, Seg b, Seg c, float scale) {
   const int total = a.len + b.len + c.len;
-  k_gnn_reduce<<<(total + 31) / 32, NB, 0, md->s>>>(md->part, nblk, stride, a, b, c, md->grad,
+  k_gnn_reduce<<<(total + 31) / 32, kReduceNB, 0, md->s>>>(md->part, nblk, stride, a, b, c, md->grad,
                                                         scale);
   GTRY(cudaGetLastError());
   return PDLP_OK;
@@ -1168,12 +1341,12 @@ int backward(gnn_model* md, gnn_graph* g, float scale) {
   const int Gs = sm_count() * 8, Gb = sm_count() * 2;
   // heads (with dH) -- their partials are reduced right after each head
   RTRY(forward(md, g, false, true, true));
-  const int gx = grid_rows((long long)n, 16, md->max_blocks);
-  const int gy = grid_rows((long long)m, 16, md->max_blocks);
+  const int gx = grid_rows((long long)n, kHeadRows, md->max_blocks);
+  const int gy = grid_rows((long long)m, kHeadRows, md->max_blocks);
   if (n > 0) RTRY(reduce_into(md, gx, 65, Seg{0, 64, kOff.w_x}, Seg{64, 1, kOff.b_x}, Seg{0, 0, 0}, scale));
   if (m > 0) {
     // the y head's partials sit after the x head's in md->part
-    k_gnn_reduce<<<3, NB, 0, s>>>(md->part + (size_t)gx * 65, gy, 65, Seg{0, 64, kOff.w_y},
+    k_gnn_reduce<<<3, kReduceNB, 0, s>>>(md->part + (size_t)gx * 65, gy, 65, Seg{0, 64, kOff.w_y},
                                   Seg{64, 1, kOff.b_y}, Seg{0, 0, 0}, md->grad, scale);
     GTRY(cudaGetLastError());
   }
@@ -1190,8 +1363,8 @@ int backward(gnn_model* md, gnn_graph* g, float scale) {
                        Seg{8192, 64, kOff.b_v[k]}, scale));
       if (m > 0) {
         // dH_c += C dS_v, C_ij = a_ij / deg_j
-        k_gnn_spmm<<<grid_rows((long long)m, NB / 16, Gs), NB, 0, s>>>(
-            m, g->d.a_ptr, g->d.a_col, g->d.a_val, nullptr, g->inv_deg_c, md->dsv, md->dhc[cur], 1);
+        k_gnn_spmm<<<grid_rows((long long)m, NB / 16, kAnyGrid), NB, 0, s>>>(
+            m, g->d.a_ptr, g->d.a_col, g->a_v32, nullptr, g->inv_deg_c, md->dsv, md->dhc[cur], 1);
         GTRY(cudaGetLastError());
       }
     }
@@ -1205,22 +1378,22 @@ int backward(gnn_model* md, gnn_graph* g, float scale) {
                        Seg{8192, 64, kOff.b_c[k]}, scale));
       if (n > 0) {
         // dH_v += R^T dS_c, R_ij = a_ij / deg_i
-        k_gnn_spmm<<<grid_rows((long long)n, NB / 16, Gs), NB, 0, s>>>(
-            n, g->d.t_ptr, g->d.t_col, g->d.t_val, nullptr, g->inv_deg_r, md->dsc, md->dhv[nxt], 1);
+        k_gnn_spmm<<<grid_rows((long long)n, NB / 16, kAnyGrid), NB, 0, s>>>(
+            n, g->d.t_ptr, g->d.t_col, g->t_v32, nullptr, g->inv_deg_r, md->dsc, md->dhv[nxt], 1);
         GTRY(cudaGetLastError());
       }
     }
     cur = nxt;
   }
   if (n > 0) {
-    const int ge = grid_rows((long long)n, 4, Gb);
+    const int ge = grid_rows((long long)n, 4, Gs);
     k_gnn_embed_bwd<GNN_VAR_FEATURES><<<ge, NB, 0, s>>>(n, g->fv, md->hv[0], md->dhv[cur], md->part);
     GTRY(cudaGetLastError());
     RTRY(reduce_into(md, ge, (GNN_VAR_FEATURES + 1) * H, Seg{0, GNN_VAR_FEATURES * H, kOff.W_vin},
                      Seg{GNN_VAR_FEATURES * H, H, kOff.b_vin}, Seg{0, 0, 0}, scale));
   }
   if (m > 0) {
-    const int ge = grid_rows((long long)m, 4, Gb);
+    const int ge = grid_rows((long long)m, 4, Gs);
     k_gnn_embed_bwd<GNN_CON_FEATURES><<<ge, NB, 0, s>>>(m, g->fc, md->hc[0], md->dhc[cur], md->part);
     GTRY(cudaGetLastError());
     RTRY(reduce_into(md, ge, (GNN_CON_FEATURES + 1) * H, Seg{0, GNN_CON_FEATURES * H, kOff.W_cin},
@@ -1277,11 +1450,9 @@ int gnn_create(uint64_t seed, gnn_model** out) {
     return bail(gfail(PDLP_ERR_OOM, "model allocation failed"));
   const size_t part_floats = std::max<size_t>((size_t)sm_count() * 2 * kDensePart,
                                               (size_t)2 * md->max_blocks * 65);
-  if (dalloc(&md->part, std::max<size_t>(part_floats, (size_t)sm_count() * 2 * 7 * H)) != cudaSuccess)
+  if (dalloc(&md->part, std::max<size_t>(part_floats, (size_t)sm_count() * 8 * 7 * H)) != cudaSuccess)
     return bail(gfail(PDLP_ERR_OOM, "model allocation failed"));
-  e = cudaFuncSetAttribute(k_gnn_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gnn_dense_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmem);
+  e = cudaFuncSetAttribute(k_gnn_dense_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmem);
   if (e != cudaSuccess) return bail(gfail(PDLP_ERR_CUDA, cudaGetErrorString(e)));
   // Xavier-uniform from SplitMix64, block by block in parameter order
   std::vector<float> th(md->P, 0.f);
@@ -1428,7 +1599,9 @@ int gnn_graph_create(gnn_model* md, const pdlp_csr* A, const double* b, const ch
   // the graph's own arrays and the feature pass's scratch share the LP's allocation
   const size_t M = A ? (size_t)std::max(A->m, 0) : 0, N = A ? (size_t)std::max(A->n, 0) : 0;
   Carve cv;
+  const size_t Z = A ? (size_t)std::max<int64_t>(A->nnz, 0) : 0;
   const size_t o_idr = cv.take(4 * M), o_idc = cv.take(4 * N);
+  const size_t o_av = cv.take(4 * Z), o_tv = cv.take(4 * Z);
   const size_t o_fv = cv.take(4 * N * GNN_VAR_FEATURES), o_fc = cv.take(4 * M * GNN_CON_FEATURES);
   const size_t o_nr = cv.take(8 * M), o_nc = cv.take(8 * N), o_mx = cv.take(6 * 8);
   int rc = build_lp_dev(A, b, sense, c, l, u, s, &g->d, cv.off);
@@ -1440,6 +1613,8 @@ int gnn_graph_create(gnn_model* md, const pdlp_csr* A, const double* b, const ch
   unsigned char* ex = g->d.extra;
   g->inv_deg_r = (float*)(ex + o_idr);
   g->inv_deg_c = (float*)(ex + o_idc);
+  g->a_v32 = (float*)(ex + o_av);
+  g->t_v32 = (float*)(ex + o_tv);
   g->fv = (float*)(ex + o_fv);
   g->fc = (float*)(ex + o_fc);
   double* nr = (double*)(ex + o_nr);
@@ -1448,6 +1623,11 @@ int gnn_graph_create(gnn_model* md, const pdlp_csr* A, const double* b, const ch
   unsigned long long hmx[6] = {};
   cudaError_t e = cudaMemsetAsync(mx, 0, 6 * sizeof(unsigned long long), s);
   const int G = sm_count() * 8;
+  if (e == cudaSuccess && g->d.nnz > 0) {
+    k_gnn_values<<<grid_rows(g->d.nnz, NB, G), NB, 0, s>>>(g->d.nnz, g->d.a_val, g->d.t_val, g->a_v32,
+                                                           g->t_v32);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess && m > 0) {
     k_gnn_stats<<<grid_rows(m, NB, G), NB, 0, s>>>(m, g->d.a_ptr, g->d.a_val, g->d.b, nr,
                                                    g->inv_deg_r, mx);
