@@ -235,7 +235,16 @@ cudaError_t launch_persist_t(int lanes_a, int lanes_t, const IterRaw& r, int max
       allowed_dev = dev;
     }
     if (grid_out) *grid_out = 1;
-    kern<<<1, kBlock, r.smem.bytes, s>>>(d, r.smem, max_attempts);
+    // threads for one round of the longer side, lanes for what a side leaves over
+    const int side = r.m > r.n ? r.m : r.n;
+    int threads = 256;
+    while (threads < SmemThreads<T>::value && threads < side) threads <<= 1;
+    auto lanes = [&](int rows) {
+      int L = 1;
+      while (L < 8 && 2 * L * rows <= threads) L <<= 1;
+      return L;
+    };
+    kern<<<1, threads, r.smem.bytes, s>>>(d, r.smem, lanes(r.n), lanes(r.m), max_attempts);
     return cudaGetLastError();
   }
   switch (lanes_a) {

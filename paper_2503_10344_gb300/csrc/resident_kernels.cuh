@@ -189,28 +189,39 @@ __device__ __forceinline__ float div_pos(float n, float d) {
   return fmaf(fmaf(-q, d, n), r, q);
 }
 
-// Sum over a warp whose lanes other than the multiples of `step` (a power of two) below `used`
-// hold zeros, in every lane that is such a multiple (lane 0 among them): the levels that would add
-// zeros only are left out, and all of them where every lane holds zero (rows that did not move,
-// warps without rows).  In float64 a level costs a warp some 16 cycles of the SM's one pipe; in
-// float32 the tests would cost more than the levels, and all are added.
-template <typename T>
-__device__ __forceinline__ T res_warp_sum(T v, int step, int used) {
-  if constexpr (std::is_same<T, float>::value) return group_sum<32>(v);
-  if (!__any_sync(0xffffffffu, v != (T)0)) return (T)0;
-  for (int o = 16; o >= step; o >>= 1) {
-    const T w = __shfl_xor_sync(0xffffffffu, v, o);
-    if (o < used) v += w;
+// N sums over a warp whose lanes other than the multiples of `step` (a power of two) below `used`
+// hold zeros, in every lane that is such a multiple (lane 0 among them).  In float64, where an
+// addition takes some 100 cycles and holds the SM's one pipe for 16, the levels that would add zeros
+// only are left out, and all of them where every lane holds zeros (rows that did not move, warps
+// without rows); in float32 the tests would cost more than the levels.  The sums advance level by
+// level together: shuffles stay in program order, so sum after sum waits for each addition.
+template <int N, typename T>
+__device__ __forceinline__ void res_warp_sums(T (&v)[N], int step, int used) {
+  constexpr bool F64 = std::is_same<T, double>::value;
+  if constexpr (F64) {
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < N; ++k) any |= __double_as_longlong(v[k]) << 1 != 0;  // (not +0, not -0)
+    if (!__any_sync(0xffffffffu, any)) return;
   }
-  return v;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (F64 && (o < step || o >= used)) continue;
+    T w[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) w[k] = __shfl_xor_sync(0xffffffffu, v[k], o);
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] += w[k];
+  }
 }
 
 // This block's three sums (of lane 0) posted to every replica under `tag`, and the sums over
 // all blocks in slot order per lane, then a fixed shuffle tree (in lane 0).  Called by one whole warp.
 // (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.)
-template <typename T>
+// `meanwhile` runs between the posting and the polling.
+template <typename T, typename F>
 __device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* slot, int G,
-                                         unsigned tag, int limit, T (&sum)[3]) {
+                                         unsigned tag, int limit, T (&sum)[3], F meanwhile) {
   using S = ResS<T>;
   constexpr int reps = res_replicas((int)sizeof(T)), kPoll = sizeof(T) == 8 ? 2 : kResPoll;
   const int lane = threadIdx.x & 31, b = blockIdx.x;
@@ -218,6 +229,7 @@ __device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* s
 #pragma unroll
     for (int k = 0; k < 3; ++k) sum[k] = __shfl_sync(0xffffffffu, sum[k], 0);
   if (lane < reps) S::post(slot + (size_t)lane * G + b, sum, tag);
+  meanwhile();
   const typename S::Word* mine = slot + (size_t)(b % reps) * G;
   bool ok = true;
   sum[0] = sum[1] = sum[2] = (T)0;
@@ -249,8 +261,7 @@ __device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* s
       }
   }
   ok = __all_sync(0xffffffffu, ok);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) sum[k] = res_warp_sum<T>(sum[k], 1, G);
+  res_warp_sums(sum, 1, G);
   return ok;
 }
 
@@ -427,21 +438,23 @@ __device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
 }
 
 // The step decision (decide_step, the same operations in the iterate type) in two halves: what the
-// next attempt reads, which every thread of the block waits for, and the rest of the state, which
-// the deciding thread writes while the others go on.
+// next attempt reads, which every thread of the block waits for, and the rest of the state, written
+// later in the shadow of something else (700-970 cycles of a thread that nobody waits for; at the
+// start of the next attempt they delayed its whole block: a tenth of an attempt).
 template <typename T>
 struct ResDecision {
   T eta, eta_bar, eta_next;
-  bool accept;
+  bool accept, numerical;
 };
 template <typename T>
 __device__ __forceinline__ ResDecision<T> res_decide(DevState* st, T dx2, T dy2, T dkd, T fd, T fi,
                                                      int& left) {
   constexpr bool F64 = std::is_same<T, double>::value;
   const T eta = F64 ? (T)st->eta : (T)st->eta_f;
-  ResDecision<T> r{eta, (T)INFINITY, eta, true};
+  ResDecision<T> r{eta, (T)INFINITY, eta, true, false};
   if (!isfinite(dx2) || !isfinite(dy2) || !isfinite(dkd)) {
     st->status = 4;  // PDLP_NUMERICAL
+    r.numerical = true;
     return r;
   }
   const T om = F64 ? (T)st->omega : (T)st->omega_f, iom = F64 ? (T)0 : (T)st->inv_omega_f;
@@ -479,7 +492,7 @@ template <typename T>
 __device__ __forceinline__ void res_record(DevState* st, const ResDecision<T>& r) {
   const long long t = st->attempts;
   st->attempts = t + 1;
-  if (st->status == 4) return;
+  if (r.numerical) return;
   if (t < st->tr_cap) {
     st->tr_eta[t] = (double)r.eta;
     st->tr_eta_bar[t] = (double)r.eta_bar;
@@ -612,6 +625,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
   const int ahead_n = nt ? tp[res_chunk_end(tp, nt, R.cap_t, 0)] : 0;  // the first chunk of st
   const ResWait wait{gst, (int)ls.spin_limit, 0};
   ResDecision<T> dec{};
+  const long long first_attempt = ls.attempts;
   unsigned ytag = tag0 + 1u;
   bool ahead = false;  // the first chunk of the next primal step is staged
   for (int att = 0; att < max_attempts; ++att) {
@@ -619,10 +633,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
     const T pw = StepT<T>::pw(&ls), tau = StepT<T>::tau(&ls), sigma = StepT<T>::sigma(&ls);
     const unsigned tag = tag0 + 2u * (unsigned)(att + 1);
     T fd = 0, fi = 0;
-    if (tid == 0) {
-      if (att > 0) res_record(&ls, dec);  // of the attempt before
-      step_factors(&ls, ls.attempts + 1, &fd, &fi);
-    }
+    if (tid == 0) step_factors(&ls, first_attempt + att + 1, &fd, &fi);
     // ---- A4: primal step over the block's columns
     {
       const T* xo = xs[cur];
@@ -641,8 +652,9 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         else dx2 += dd * dd;
       };
       res_product<T, EY>(R.lanes_t, st, ex_y(cur), ytag, stage1, ahead, wait, &fail, fin);
-      dx2 = res_warp_sum<T>(dx2, R.lanes_t, 32);
-      if ((tid & 31) == 0) red[0][tid >> 5] = dx2;
+      T v[1] = {dx2};
+      res_warp_sums(v, R.lanes_t, 32);
+      if ((tid & 31) == 0) red[0][tid >> 5] = v[0];
     }
     __syncthreads();  // the stage is free
     // ---- A5: dual step over the block's rows
@@ -666,20 +678,27 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         dkd += dd * acc.b;
       };
       res_product<T, EX>(R.lanes_a, sa, ex_x, tag, stage2, false, wait, &fail, fin);
-      dy2 = res_warp_sum<T>(dy2, R.lanes_a, 32);
-      dkd = res_warp_sum<T>(dkd, R.lanes_a, 32);
+      T v[2] = {dy2, dkd};
+      res_warp_sums(v, R.lanes_a, 32);
       if ((tid & 31) == 0) {
-        red[1][tid >> 5] = dy2;
-        red[2][tid >> 5] = dkd;
+        red[1][tid >> 5] = v[0];
+        red[2][tid >> 5] = v[1];
       }
     }
     __syncthreads();  // the stage is free, the warps' sums are there
     if (tid < 32) {
       T s[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) s[k] = res_warp_sum<T>(red[k][tid], 1, NT >> 5);
+      for (int k = 0; k < 3; ++k) s[k] = red[k][tid];
+      res_warp_sums(s, 1, NT >> 5);
       bool ok = fail == 0;
-      if (G > 1) ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, G, tag, wait.limit, s) && ok;
+      auto record = [&] {  // of the attempt before, while the sums travel
+        if (tid == 0 && att > 0) res_record(&ls, dec);
+      };
+      if (G > 1)
+        ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, G, tag, wait.limit, s, record) && ok;
+      else
+        record();
       // ---- A6: the same decision in every block
       if (tid == 0) {
         dec = res_decide<T>(&ls, s[0], s[1], s[2], fd, fi, left);

@@ -528,33 +528,33 @@ struct SetupOut {
 };
 
 // The form of the step attempts of one LP where the caller asks for none (persistent = 0 without
-// lanes, tiles, the autotuner or the Halpern variant): with float32 iterates the LP in one block's
-// shared memory up to kOneBlockNnz nonzeros; spread over the SMs' shared memory
+// lanes, tiles, the autotuner or the Halpern variant): the LP in one block's shared memory up to
+// one_block_nnz() nonzeros; spread over the SMs' shared memory
 // (resident_kernels.cuh) while it fits there, else three launches per attempt.  Measured per
 // attempt on a GB300 (us; values in float32 / bfloat16 or the 0/1 pattern):
 //                                 nonzeros   three launches   one block     resident
-//   relaxation 200 x 400             1,670      9.9 /  9.4    2.5 /  2.8    3.8 /  3.7
-//   relaxation 400 x 800             3,238     10.0 /  9.6    3.9 /  4.6    3.7 /  3.7
-//   relaxation 2,000 x 4,000        15,963     13.4 / 12.0   30.3 / 36.4    4.4 /  4.5
-//   covering 2,000 x 8,000          54,130     12.4 / 11.6                  5.0 /  5.0
-//   covering 10,000 x 40,000       269,989     14.2 / 13.0                  6.6 /  6.4
-//   covering 50,000 x 200,000    1,350,409     23.0 / 20.5                 20.3 / 13.7
-//   energy system, 24 h             21,600     23.3                         4.9
-//   energy system, 720 h           648,000     17.7                        10.4
-// and in float64 (one block would win nothing: its chains of float64 operations are as long):
-//   relaxation 40 x 80                 320     15.5             6.4           5.6
-//   relaxation 200 x 400             1,670     16.6             7.7           7.9
-//   relaxation 2,000 x 4,000        15,963     19.1                           8.7
-//   covering 2,000 x 8,000          54,130     25.8                          10.4
-//   covering 10,000 x 40,000       269,989     33.7                          14.4
-//   covering 25,000 x 100,000      675,211     40.0                          27.7
-//   energy system, 24 h             21,600     23.7                          10.8
-//   energy system, 400 h           360,000    129.0                          18.5
+//   relaxation 200 x 400             1,670      9.9 /  9.4    2.1 /  2.2    3.5 /  3.3
+//   relaxation 400 x 800             3,238     10.0 /  9.6    2.8           3.5
+//   relaxation 2,000 x 4,000        15,963     13.4 / 12.0   30.3 / 36.4          3.8
+//   covering 2,000 x 8,000          54,130     12.4 / 11.6                        4.1
+//   covering 10,000 x 40,000       269,989     14.2 / 13.0                        5.6
+//   covering 50,000 x 200,000    1,350,409     23.0 / 20.5                 20.3 / 12.8
+//   energy system, 24 h             21,600     23.3                         4.4
+//   energy system, 720 h           648,000     17.7                         9.9
+// and in float64 (the one block's chains of float64 operations are about as long as the exchange):
+//   relaxation 40 x 80                 320     15.5             4.1           5.0
+//   relaxation 200 x 400             1,670     16.6             6.6           6.6
+//   relaxation 2,000 x 4,000        15,963     19.1                           7.6
+//   covering 2,000 x 8,000          54,130     25.8                           9.0
+//   covering 10,000 x 40,000       269,989     33.7                          13.2
+//   covering 25,000 x 100,000      675,211     40.0                          25.7
+//   energy system, 24 h             21,600     23.7                          10.0
+//   energy system, 400 h           360,000    129.0                          17.6
 // kResNnz nonzeros per block: 256 and 1,024 measured within 10 % of 512, slower on most; in
 // float64 256 (128: 3-6 % slower, 512: 2 % faster to 10 % slower).
 constexpr int kResNnz = 512, kResNnz64 = 256;
-constexpr int kOneBlockNnz = 2500;
-static int one_block_nnz(Mode mode) { return mode == MODE_FP64 ? 0 : kOneBlockNnz; }
+constexpr int kOneBlockNnz = 2500, kOneBlockNnz64 = 1000;
+static int one_block_nnz(Mode mode) { return mode == MODE_FP64 ? kOneBlockNnz64 : kOneBlockNnz; }
 // Float64 solves that record iterates or decisions are parity runs against a reference: they keep
 // the separate launches, whose order of summation such records were made with.
 static bool parity_run(Mode mode, const pdlp_diagnostics* dg) {
@@ -1295,7 +1295,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     }
   }
   // one block: asked for, or a small LP whose form is ours to choose (and which fits: below)
-  const bool small = auto_form(p, m, nnz) && nnz <= one_block_nnz(mode) &&
+  const bool small = auto_form(p, m, nnz) && nnz <= one_block_nnz(mode) && !parity_run(mode, dg) &&
                      smem_layout(m, n, nnz, mode == MODE_FP64 ? 8 : 4, mode != MODE_PAT,
                                  mode == MODE_BF16 || mode == MODE_PAT).bytes <=
                          optin_smem() - kSmemStatic;
