@@ -130,6 +130,7 @@ struct ResPlan {
   int bits_t, bits_a;          // bits of an index of a gather (the rest of its word: the place)
   int shift_t, shift_a;        // index >> shift: the bucket it is ordered by
   int cap_t, cap_a;            // nonzeros staged at a time
+  int global_values;           // 1: the values stay in global memory (float64)
 };
 
 struct IterRaw {

@@ -183,10 +183,10 @@ cudaError_t launch_persist_la(int lanes_t, const IterData<T, V>& d, int max_atte
 
 // The resident step kernel: one cooperative launch of r.res.G blocks, at most one per SM.
 // max_attempts = 0 launches nothing and answers whether a block fits on an SM.
-template <typename T, typename V, bool IMPLICIT>
+template <typename T, typename V, bool IMPLICIT, bool GV = false>
 cudaError_t launch_resident_t(const IterRaw& r, int max_attempts, cudaStream_t s) {
   const IterData<T, V> d = typed<T, V>(r);
-  auto kern = k_resident<T, V, IMPLICIT>;
+  auto kern = k_resident<T, V, IMPLICIT, GV>;
   // its dynamic shared memory: a property of the kernel on this device, so every launch sets
   // the same value, the largest (a launch of another thread may be in between)
   int dev = 0, optin = 0;

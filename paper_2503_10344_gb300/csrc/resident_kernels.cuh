@@ -270,7 +270,8 @@ template <typename V>
 struct ResSide {
   const int* ptr;       // [rows + 1] relative to the block's first nonzero
   const unsigned* key;  // [nnz] the gathers: index | (place in the chunk << bits)
-  const V* val;         // [nnz] values in storage order (none for a pattern)
+  const V* val;         // [nnz] values in storage order (none for a pattern); with GV in global
+                        // memory, staged with the entries that they multiply
   const int* lng;       // [nlong] rows longer than kResLong
   int rows, nlong, bits, cap;
 };
@@ -337,11 +338,11 @@ __device__ __forceinline__ void res_sort_keys(const int* __restrict__ col, int n
 // Sums over the staged entries of rows [ra, rb) of the chunk that starts at nonzero p0, and
 // their epilogues: LANES lanes per row, then a warp per long row.
 template <int LANES, typename T, typename Acc, typename V, typename Fin>
-__device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, int p0, int ra,
-                                         int rb, Fin fin) {
+__device__ __forceinline__ void res_rows(const ResSide<V>& s, const V* val, const Acc* stage, int p0,
+                                         int ra, int rb, Fin fin) {
   const int lane = threadIdx.x & (LANES - 1), NT = blockDim.x;
   auto add = [&](Acc& acc, int p) {
-    const T v = res_val<T, V>(s.val, p);
+    const T v = res_val<T, V>(val, p);
     const Acc t = stage[p - p0];
     if constexpr (std::is_same<Acc, T>::value) acc += v * t;
     else acc += Acc{v * t.a, v * t.b};
@@ -369,14 +370,14 @@ __device__ __forceinline__ void res_rows(const ResSide<V>& s, const Acc* stage, 
 }
 
 template <typename T, typename Acc, typename V, typename Fin>
-__device__ __forceinline__ void res_rows_lanes(int lanes, const ResSide<V>& s, const Acc* stage,
-                                               int p0, int ra, int rb, Fin fin) {
+__device__ __forceinline__ void res_rows_lanes(int lanes, const ResSide<V>& s, const V* val,
+                                               const Acc* stage, int p0, int ra, int rb, Fin fin) {
   switch (lanes) {
-    case 1: return res_rows<1, T>(s, stage, p0, ra, rb, fin);
-    case 2: return res_rows<2, T>(s, stage, p0, ra, rb, fin);
-    case 4: return res_rows<4, T>(s, stage, p0, ra, rb, fin);
-    case 8: return res_rows<8, T>(s, stage, p0, ra, rb, fin);
-    default: return res_rows<16, T>(s, stage, p0, ra, rb, fin);
+    case 1: return res_rows<1, T>(s, val, stage, p0, ra, rb, fin);
+    case 2: return res_rows<2, T>(s, val, stage, p0, ra, rb, fin);
+    case 4: return res_rows<4, T>(s, val, stage, p0, ra, rb, fin);
+    case 8: return res_rows<8, T>(s, val, stage, p0, ra, rb, fin);
+    default: return res_rows<16, T>(s, val, stage, p0, ra, rb, fin);
   }
 }
 
@@ -384,11 +385,16 @@ __device__ __forceinline__ void res_rows_lanes(int lanes, const ResSide<V>& s, c
 // block, E::kInFlight loads in flight each.  Returns false when a wait gave up.
 // (A newer tag ends the wait too: only the y gathered ahead of a step that is then rejected can
 // meet one, and it is dropped.)
-template <typename E, typename V>
+template <bool GV, typename E, typename V>
 __device__ __forceinline__ bool res_gather(const ResSide<V>& s, int p0, int n,
                                            const typename E::Word* __restrict__ from, unsigned tag,
                                            typename E::Acc* stage, int t, int nt, ResWait wait) {
   constexpr int U = E::kInFlight;
+  if constexpr (GV) {  // the chunk's values, behind its entries
+    V* vst = (V*)(stage + s.cap);
+#pragma unroll 4
+    for (int i = t; i < n; i += nt) vst[i] = __ldg(s.val + p0 + i);
+  }
   const unsigned mask = (1u << s.bits) - 1u;
   const unsigned* key = s.key + p0;
   for (int i0 = t; i0 < n; i0 += nt * U) {
@@ -419,7 +425,7 @@ __device__ __forceinline__ bool res_gather(const ResSide<V>& s, int p0, int n,
 
 // A side's product: chunk by chunk the entries its rows need, then the rows' sums.  The first
 // chunk may have been gathered ahead (`ahead`).
-template <typename T, typename E, typename V, typename Fin>
+template <typename T, bool GV, typename E, typename V, typename Fin>
 __device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
                                             const typename E::Word* from, unsigned tag,
                                             typename E::Acc* stage, bool ahead, ResWait wait,
@@ -429,10 +435,10 @@ __device__ __forceinline__ void res_product(int lanes, const ResSide<V>& s,
     const int p0 = s.ptr[ra], rb = res_chunk_end(s.ptr, s.rows, s.cap, ra);
     if (ra > 0) __syncthreads();  // the chunk before is summed
     if (ra > 0 || !ahead)
-      if (!res_gather<E>(s, p0, s.ptr[rb] - p0, from, tag, stage, threadIdx.x, blockDim.x, wait))
+      if (!res_gather<GV, E>(s, p0, s.ptr[rb] - p0, from, tag, stage, threadIdx.x, blockDim.x, wait))
         *fail = 1;
     __syncthreads();
-    res_rows_lanes<T, typename E::Acc>(lanes, s, stage, p0, ra, rb, fin);
+    res_rows_lanes<T, typename E::Acc>(lanes, s, GV ? (const V*)(stage + s.cap) - p0 : s.val, stage, p0, ra, rb, fin);
     ra = rb;
   }
 }
@@ -508,7 +514,8 @@ __device__ __forceinline__ void res_record(DevState* st, const ResDecision<T>& r
   }
 }
 
-template <typename T, typename V, bool IMPLICIT>
+// GV: the matrix values stay in global memory (L2) and are copied with each chunk.
+template <typename T, typename V, bool IMPLICIT, bool GV>
 __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, ResPlan R,
                                                            int max_attempts) {
   using EY = ResY<T>;
@@ -534,7 +541,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
   const int nt = t1 - t0, na = a1 - a0;
   const int tz0 = __ldg(d.t_ptr + t0), az0 = __ldg(d.a_ptr + a0);
   const int tz = __ldg(d.t_ptr + t1) - tz0, az = __ldg(d.a_ptr + a1) - az0;
-  const ResLayout L = res_layout(nt, tz, na, az, (int)sizeof(T), VALS ? (int)sizeof(V) : 0, IMPLICIT);
+  const ResLayout L = res_layout(nt, tz, na, az, (int)sizeof(T), VALS && !GV ? (int)sizeof(V) : 0, IMPLICIT);
   int* tp = (int*)(sm + L.t_ptr);
   unsigned* tk = (unsigned*)(sm + L.t_col);
   V* tv = VALS ? (V*)(sm + L.t_val) : nullptr;
@@ -581,7 +588,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
     xs[cur0][j] = d.x[cur0][t0 + j].x;
     sx[j] = d.sum_x[t0 + j];
   }
-  if constexpr (VALS) {
+  if constexpr (VALS && !GV) {
     for (int p = tid; p < tz; p += NT) tv[p] = d.t_val[tz0 + p];
     for (int p = tid; p < az; p += NT) av[p] = d.a_val[az0 + p];
   }
@@ -620,8 +627,8 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
     left = (int)(p < q ? p : q > 1 ? q : 1);
   }
   __syncthreads();
-  const ResSide<V> st{tp, tk, tv, tl, nt, nlong[0], R.bits_t, R.cap_t};
-  const ResSide<V> sa{ap, ak, av, al, na, nlong[1], R.bits_a, R.cap_a};
+  const ResSide<V> st{tp, tk, GV ? d.t_val + tz0 : tv, tl, nt, nlong[0], R.bits_t, R.cap_t};
+  const ResSide<V> sa{ap, ak, GV ? d.a_val + az0 : av, al, na, nlong[1], R.bits_a, R.cap_a};
   const int ahead_n = nt ? tp[res_chunk_end(tp, nt, R.cap_t, 0)] : 0;  // the first chunk of st
   const ResWait wait{gst, (int)ls.spin_limit, 0};
   ResDecision<T> dec{};
@@ -651,7 +658,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         if constexpr (IMPLICIT) dx2 += div_pos(dd * dd, w);
         else dx2 += dd * dd;
       };
-      res_product<T, EY>(R.lanes_t, st, ex_y(cur), ytag, stage1, ahead, wait, &fail, fin);
+      res_product<T, GV, EY>(R.lanes_t, st, ex_y(cur), ytag, stage1, ahead, wait, &fail, fin);
       T v[1] = {dx2};
       res_warp_sums(v, R.lanes_t, 32);
       if ((tid & 31) == 0) red[0][tid >> 5] = v[0];
@@ -677,7 +684,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         else dy2 += dd * dd;
         dkd += dd * acc.b;
       };
-      res_product<T, EX>(R.lanes_a, sa, ex_x, tag, stage2, false, wait, &fail, fin);
+      res_product<T, GV, EX>(R.lanes_a, sa, ex_x, tag, stage2, false, wait, &fail, fin);
       T v[2] = {dy2, dkd};
       res_warp_sums(v, R.lanes_a, 32);
       if ((tid & 31) == 0) {
@@ -704,7 +711,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         dec = res_decide<T>(&ls, s[0], s[1], s[2], fd, fi, left);
         stop = !ok ? 2 : (ls.status != 0 || ls.check_due) ? 1 : 0;
       }
-    } else if (!res_gather<EY>(st, 0, ahead_n, ex_y(cur ^ 1), tag, stage1, tid - 32, NT - 32,
+    } else if (!res_gather<GV, EY>(st, 0, ahead_n, ex_y(cur ^ 1), tag, stage1, tid - 32, NT - 32,
                                  wait)) {
       fail = 1;
     }

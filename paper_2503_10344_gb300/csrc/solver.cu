@@ -524,6 +524,7 @@ struct SetupOut {
   int tiles, n_ta, n_tt;  // staged tile kernels built; their items over A and A^T
   int res_G;              // blocks of the resident step kernel (0: not planned)
   ResBufs rb;             // its buffers
+  int res_gv;             // its matrix values stay in global memory
   ResSizes res;
 };
 
@@ -686,13 +687,23 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
   // buffers in scratch that is free by now: the scalars' partial sums or the transpose's, and in
   // float64, where they are twice as large, those and the scaling's statistics and the step
   // weights of the other storage form
-  so->res_G = 0;
+  so->res_G = so->res_gv = 0;
   so->rb = ResBufs{};
   so->res = ResSizes{};
   if (auto_form(p, m, nnz) && nnz > one_block_nnz(mode) && !parity_run(mode, dg)) {
     const int it = mode == MODE_FP64 ? 8 : 4;
-    const int vb = mode == MODE_FP64 ? 8 : mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
+    int vb = mode == MODE_FP64 ? 8 : mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
     const long long data = nnz * 2 * (4 + vb) + 6LL * it * ((long long)m + n);
+    const long long chip = (long long)device_sm_count() * optin_smem();
+    const bool fits = data <= chip;
+    if (mode == MODE_FP64 && data > chip * 3 / 4) {
+      // no room left for the stage: the values are copied from L2 with each stage instead.  Per
+      // attempt against three launches: energy system 720 h 39.8 us to 132.9, covering LP 38,000 x
+      // 152,000 40.2 to 42.0; one of 50,000 x 200,000, which is more than the SMs hold with its
+      // values, 60.5 to 48.4
+      so->res_gv = 1;
+      vb = 0;
+    }
     const int G = resident_blocks(mode, nnz);
     const Region part{bf.part_setup, 8 * setup_part_doubles(m, n)}, tmp{bf.tmp, bf.tmp_bytes};
     if (mode == MODE_FP64) {
@@ -706,7 +717,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
       so->rb.place(&tmp, 1, G, m, n, it);
     }
     const ResBufs& rb = so->rb;
-    if (rb.ok && data <= (long long)device_sm_count() * optin_smem()) {
+    if (rb.ok && fits) {
       so->res_G = G;
       CUDA_TRY(setup_res_plan(m, n, (int)nnz, bf.a_ptr, bf.t_ptr, G, it, vb,
                               mode == MODE_BF16 || mode == MODE_PAT, rb.cut_t, rb.cut_a, rb.sizes, s));
@@ -1276,13 +1287,15 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     R.lanes_a = lanes(z.a_rows, (double)nnz / m);
     // the stage: a side's whole part where it fits, else as much as does (whole rows)
     const long long room = optin_smem() - kSmemStatic - (long long)z.bytes;
+    R.global_values = so.res_gv;
+    const int et = it * (so.res_gv ? 2 : 1), ea = it * (so.res_gv ? 3 : 2);  // bytes staged per entry
     const long long want =
-        (std::max({(long long)it * z.t_nnz, 2LL * it * z.a_nnz, 4LL * kResBuckets}) + 15) / 16 * 16;
+        (std::max({(long long)et * z.t_nnz, (long long)ea * z.a_nnz, 4LL * kResBuckets}) + 15) / 16 * 16;
     const long long stage = std::min(want, room / 16 * 16);
-    R.cap_t = (int)(stage / it);
-    R.cap_a = (int)(stage / (2 * it));
+    R.cap_t = (int)(stage / et);
+    R.cap_a = (int)(stage / ea);
     R.smem = (int)(z.bytes + stage);
-    const bool fits = stage == want || stage >= 2LL * it * std::max(z.max_len, kResMinStage);
+    const bool fits = stage == want || stage >= (long long)ea * std::max(z.max_len, kResMinStage);
     if (fits && R.bits_t + bits(z.t_nnz) <= 32 && R.bits_a + bits(z.a_nnz) <= 32) {
       sv.ir.res = R;
       sv.persist_grid = R.G;

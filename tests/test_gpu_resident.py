@@ -108,6 +108,17 @@ def test_several_stages(P):
         assert rel(it[k], it0[k]) <= F32, (k, rel(it[k], it0[k]))
 
 
+def test_float64_values_from_global_memory(P):
+    """A part of the LP with its stage is more than an SM holds: the float64 values stay in global
+    memory and are staged, with the entries they multiply, in several goes."""
+    lp = lpgen.set_cover(9, m=36000, n=144000)
+    kw = dict(FIXED, iter_limit=20)
+    x, y, r = P.pdlp_solve(lp, P.default_params(**kw))
+    x0, y0, r0 = P.pdlp_solve(lp, P.default_params(lanes_A=8, lanes_AT=2, **kw))
+    assert r["persistent_form"] == 4 and r0["persistent_form"] == 0
+    assert rel(x, x0) <= F64 and rel(y, y0) <= F64
+
+
 def test_rejected_steps_float64(P):
     """As below; a rounding grows about tenfold every 40 adaptive steps, 1e-9 after 100."""
     lp = lpgen.set_cover(5, m=1500, n=6000)
@@ -138,6 +149,7 @@ def test_form_by_size(P):
     small, mid = lpgen.mip_relaxation(1), lpgen.set_cover(7, m=2000, n=8000)
     assert form(small, precision="fp32") == 3 and form(mid, precision="fp32") == 4
     assert form(small, precision="fp64") == form(mid, precision="fp64") == 4
+    assert form(lpgen.mip_relaxation(3, m=60, n=120, density=4 / 60), precision="fp64") == 3
     assert form(lpgen.set_cover(2025), precision="fp64") == 0  # more than the SMs hold
     for kw in (dict(precision="fp64", lanes_A=2), dict(precision="fp32", lanes_A=2), dict(precision="bf16", autotune=1),
                dict(precision="fp32", tiles=1), dict(precision="fp32", halpern=1)):
