@@ -233,9 +233,13 @@ static int step_lanes(double avg_len, double per_lane, bool one_ok) {
 }
 
 // Rows longer than this go to the long-row blocks (one block per row).  With one lane
-// per row a thread walks its rows' entries one after another, so the cut-off is low.
+// per row a thread walks its rows' entries one after another, so the cut-off is low, and with two
+// or four lanes likewise: 64 entries each (at 1,024 whatever the lanes, the energy system's
+// capacity columns of up to that many hours were walked by two lanes: a float64 attempt of 1,000 h
+// took 184 us against 78 of 1,500 h, whose columns had blocks).
 static int long_thresh(int step_lanes, int kkt_lanes) {
-  return step_lanes == 1 ? 64 : std::max(1024, 128 * std::max(step_lanes, kkt_lanes));
+  const int lanes = std::max(step_lanes, kkt_lanes);
+  return step_lanes == 1 ? 64 : lanes < 8 ? 64 * lanes : std::max(1024, 128 * lanes);
 }
 
 static bool valid_lanes(int l) { return l == 2 || l == 4 || l == 8 || l == 16 || l == 32; }
