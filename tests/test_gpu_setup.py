@@ -77,3 +77,39 @@ def test_batch_scalars_and_scaling(P, count):
                                    fixed_eta=0.9))
         assert r["omega"] == pytest.approx(ref.omega, rel=1e-12)
         assert rel(x, ref.x) <= 1e-12 and rel(y, ref.y) <= 1e-12
+
+
+@pytest.mark.parametrize("m,n", [(2047, 2048), (2048, 2049), (2049, 4096), (4097, 10_240)])
+def test_prefix_sums_at_tile_edges(P, m, n):
+    """Row and column counts around the 2,048 counts of a scan's tile: one launch, two, the last
+    tile full or of one count.  Twenty float64 steps agree with the oracle's to rounding."""
+    lp = lpgen.random_sparse_lp(m, m, n, density=3.0 / m)
+    kw = dict(iter_limit=20, adaptive_step=0, restarts=0, terminate=0, fixed_eta=0.5)
+    _, _, _, it = P.pdlp_solve(lp, P.default_params(**kw), iterates=True)
+    ref = O.solve(lp, O.Params(iter_limit=20, adaptive=False, restarts=False, terminate=False, fixed_eta=0.5))
+    for k in ("x_cur", "y_cur"):
+        want = getattr(ref, k)
+        assert np.linalg.norm(it[k] - want) <= 1e-12 * max(1.0, np.linalg.norm(want)), k
+
+
+@pytest.mark.parametrize("lanes", [2, 4])
+def test_long_row_cutoff(P, lanes):
+    """Rows and columns on both sides of 64 entries per lane, the cut-off to a block per row."""
+    rng = np.random.default_rng(lanes)
+    cut, n = 64 * lanes, 900
+    lengths = np.array([cut - 1, cut, cut + 1, 1, 3] * 12)
+    m = len(lengths)
+    rows = np.repeat(np.arange(m), lengths)
+    cols = np.concatenate([rng.choice(n, k, replace=False) for k in lengths])
+    lp = lpgen._lp(m, n, rows, cols, rng.integers(1, 4, rows.size).astype(float), rng.uniform(0, 2, m),
+                   rng.choice([lpgen.SENSE_GE, lpgen.SENSE_LE, lpgen.SENSE_EQ], m),
+                   rng.uniform(-1, 1, n), np.zeros(n), rng.uniform(1, 5, n), np.zeros(n, dtype=np.uint8),
+                   f"cutoff_{lanes}")
+    kw = dict(iter_limit=20, adaptive_step=0, restarts=0, terminate=0, fixed_eta=0.5)
+    _, _, r, it = P.pdlp_solve(lp, P.default_params(lanes_A=lanes, lanes_AT=lanes, lanes_kkt_A=lanes,
+                                                    lanes_kkt_AT=lanes, **kw), iterates=True)
+    ref = O.solve(lp, O.Params(iter_limit=20, adaptive=False, restarts=False, terminate=False, fixed_eta=0.5))
+    for k in ("x_cur", "y_cur"):
+        want = getattr(ref, k)
+        assert np.linalg.norm(it[k] - want) <= 1e-12 * max(1.0, np.linalg.norm(want)), k
+    assert abs(r["rel_kkt"] - ref.kkt.rel_kkt) <= 1e-9 * ref.kkt.rel_kkt
