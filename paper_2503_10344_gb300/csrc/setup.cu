@@ -118,7 +118,10 @@ __global__ void k_scan_tiles(const int* cnt, int* out, int N, int* bsum) {
     if (i < N) out[i] = run;
     run += v[k];
   }
-  if (threadIdx.x == kBlock - 1) bsum[blockIdx.x] = sh[kBlock - 1];
+  if (threadIdx.x == kBlock - 1) {
+    bsum[blockIdx.x] = sh[kBlock - 1];
+    if (gridDim.x == 1) out[N] = sh[kBlock - 1];  // one tile: done
+  }
 }
 
 __global__ void k_scan_bsum(int* bsum, int nb, int* out, int N) {
@@ -146,9 +149,25 @@ __global__ void k_scan_bsum(int* bsum, int nb, int* out, int N) {
   if (threadIdx.x == 0) out[N] = carry;
 }
 
-__global__ void k_scan_add(int* out, int N, const int* bsum) {
+// SUMS: bsum still holds the tiles' sums, and every block adds up those before its own (the last
+// also writes the total): a launch less than scanning them first.
+template <bool SUMS>
+__global__ void __launch_bounds__(kBlock) k_scan_add(int* out, int N, const int* bsum) {
   const long long base = (long long)blockIdx.x * kScanTile;
-  const int add = bsum[blockIdx.x];
+  int add;
+  if constexpr (SUMS) {
+    __shared__ int sh[kWarps];
+    int v = 0;
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += kBlock) v += bsum[i];
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    add = 0;
+    for (int w = 0; w < kWarps; ++w) add += sh[w];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[N] = add + bsum[blockIdx.x];
+  } else {
+    add = bsum[blockIdx.x];
+  }
   for (int k = threadIdx.x; k < kScanTile; k += kBlock) {
     const long long i = base + k;
     if (i < N) out[i] += add;
@@ -807,21 +826,34 @@ cudaError_t setup_canonical(const SetupIn& in, int* a_ptr, int* a_col, double* a
   return cudaGetLastError();
 }
 
+// One launch up to kScanTile counts, two up to kScanDirect tiles (each block then reads at most
+// that many sums again), else three: a launch of the setup's many is 2-3 us (a pass of the
+// 200 x 400 relaxation, whose setup scans three times: 1,265 -> 1,215 us).
+constexpr int kScanDirect = 4096;
 cudaError_t exclusive_scan(const int* cnt, int* out, int N, int* bsum, cudaStream_t s) {
   const int nb = (N + kScanTile - 1) / kScanTile;
   if (nb > 0) {
     k_scan_tiles<<<nb, kBlock, 0, s>>>(cnt, out, N, bsum);
     RET(cudaGetLastError());
   }
+  if (nb == 1) return cudaSuccess;
+  if (nb > 1 && nb <= kScanDirect) {
+    k_scan_add<true><<<nb, kBlock, 0, s>>>(out, N, bsum);
+    return cudaGetLastError();
+  }
   k_scan_bsum<<<1, kBlock, 0, s>>>(bsum, nb, out, N);
   RET(cudaGetLastError());
   if (nb > 0) {
-    k_scan_add<<<nb, kBlock, 0, s>>>(out, N, bsum);
+    k_scan_add<false><<<nb, kBlock, 0, s>>>(out, N, bsum);
     RET(cudaGetLastError());
   }
   return cudaSuccess;
 }
 
+int scan_launches(long long N) {
+  const long long nb = (N + kScanTile - 1) / kScanTile;
+  return nb <= 1 ? 1 : nb <= kScanDirect ? 2 : 3;
+}
 size_t scan_tmp_ints(long long N) { return (size_t)((N + kScanTile - 1) / kScanTile) + 1; }
 
 cudaError_t setup_transpose(int m, int n, int nnz, const int* a_ptr, const int* a_col,

@@ -75,6 +75,7 @@ cudaError_t setup_iter_vectors(const VecIn& v, int fp32, void* c, void* l, void*
                                void* tw, void* sw, void* x0, void* y0, const int* row_of,
                                const int* a_col, const double* a_val64, int nnz, double* part,
                                double* scalars_out, cudaStream_t s);
+int scan_launches(long long N);  // of an exclusive scan of N counts
 size_t scan_tmp_ints(long long N);
 // dst[i] = src[i] + offset (index arrays moved into a batch's global numbering)
 cudaError_t setup_offset_copy(int* dst, const int* src, long long count, int offset,

@@ -633,7 +633,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
   mark("value format");
   CUDA_TRY(setup_transpose(m, n, (int)nnz, bf.a_ptr, bf.a_col, bf.a_val64, bf.t_ptr, bf.t_col,
                            t_val, bf.tmp, s, no_alloc));
-  g_launches += 13;
+  g_launches += 10 + scan_launches(n);
   mark("transpose");
   // ---- A2
   ScaleIn sc{m, n, bf.a_ptr, bf.a_col, a_val, bf.t_ptr, bf.t_col, t_val, p->ruiz_iters,
@@ -685,7 +685,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
     int* bsum = pos + R + 1;
     if (m > 0) CUDA_TRY(setup_long_rows(bf.a_ptr, m, th_a, flags, pos, bsum, bf.a_long, &nlong_a, s));
     CUDA_TRY(setup_long_rows(bf.t_ptr, n, th_t, flags, pos, bsum, bf.t_long, &nlong_t, s));
-    g_launches += 10;
+    g_launches += 4 + (m > 0 ? scan_launches(m) : 0) + scan_launches(n);
   }
   // the parts of the resident step kernel, if the LP's data can fit on the chip at all and its
   // buffers in scratch that is free by now: the scalars' partial sums or the transpose's, and in
@@ -742,7 +742,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
                          bf.tick_t, bf.tcap_t, cnt, &W, s));
     so->n_tt = cnt[0];
     so->tiles = p->tiles;
-    g_launches += 14;
+    g_launches += 2 + 2 * scan_launches(m) + 2 * scan_launches(n);
   }
   CUDA_TRY(cudaStreamSynchronize(s));  // scalars
   so->mode = mode;
@@ -2072,7 +2072,7 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
   double* t_val = mode == MODE_PAT ? nullptr : g.t_val64;
   CUDA_TRY(setup_transpose((int)M, (int)N, (int)Z, g.a_ptr, g.a_col, g.a_val64, g.t_ptr, g.t_col,
                            t_val, g.tmp, s, false));
-  g_launches += 14;
+  g_launches += 11 + scan_launches(N);
   {
     ScaleIn sc{(int)M, (int)N, g.a_ptr, g.a_col, a_val, g.t_ptr, g.t_col, t_val,
                p->ruiz_iters, p->pc_alpha, Z};
@@ -2112,7 +2112,7 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
                                    g.a_long, g.lb_a, s));
     CUDA_TRY(setup_batch_long_rows(g.t_ptr, (int)N, th_t, g.lps, count, 1, flags, pos, bsum,
                                    g.t_long, g.lb_t, s));
-    g_launches += 10;
+    g_launches += 4 + scan_launches(M) + scan_launches(N);
     std::vector<int> lb(2 * ((size_t)count + 1));
     CUDA_TRY(cudaMemcpyAsync(lb.data(), g.lb_a, 4 * ((size_t)count + 1), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaMemcpyAsync(lb.data() + count + 1, g.lb_t, 4 * ((size_t)count + 1),
@@ -2221,7 +2221,7 @@ static int solve_batch(int count, const pdlp_csr* const* A, const double* const*
                          g.tlp_a + count + 1, g.tick_a, tcap_a, ca, &W, s));
     CUDA_TRY(setup_tiles(tsh, g.t_ptr, (int)N, Z, g.row0_t, count, g.tmp, g.ti_t, g.tlp_t,
                          g.tlp_t + count + 1, g.tick_t, tcap_t, ct, &W, s));
-    g_launches += 16;
+    g_launches += 4 + 2 * scan_launches(M) + 2 * scan_launches(N);
     int bp = 0, bd = 0;
     CUDA_TRY(tile_resident_mode((Mode)mode, p->tiles, &bp, &bd));
     ir.tile = p->tiles;
