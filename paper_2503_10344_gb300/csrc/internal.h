@@ -67,7 +67,15 @@ constexpr int kResGatherY = 8;   // gathers in flight per thread: entries of y,
 constexpr int kResGatherX = 4;   // pairs
 constexpr int kResBuckets = 2048;  // buckets the gathers are ordered into
 // copies of the posted sums, by the bytes of an iterate element (a float64 slot is three words)
-__host__ __device__ constexpr int res_replicas(int it) { return it == 8 ? 8 : 16; }
+constexpr int res_replicas(int it) { return it == 8 ? 8 : 16; }
+constexpr int kResSlotSets = 2;  // sets of slots: see res_slot
+// Block b's slot in a replica for the sums posted under `tag` (two per attempt).  The sums of
+// successive attempts alternate between two sets: a block may post attempt k + 1 while another
+// still reads attempt k, but attempt k + 2 only with every block's sums of k + 1 in hand, and a
+// block posts those after it has read k.
+__host__ __device__ constexpr size_t res_slot(unsigned tag, int replicas, int replica, int G, int b) {
+  return ((size_t)(tag >> 1 & (kResSlotSets - 1)) * replicas + replica) * G + b;
+}
 constexpr int kResPoll = 5;      // slots a lane reads at a time (152 SMs: one round)
 constexpr int kResMinStage = 2048;  // nonzeros of A staged at a time at least, if not all are
 
@@ -122,7 +130,8 @@ struct ResSizes {
 struct ResPlan {
   int G;                       // blocks (0: the kernel is not used)
   const int *cut_t, *cut_a;    // [G + 1] first column / row of each block
-  void* slot;                  // [res_replicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
+  void* slot;                  // [kResSlotSets][replicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
+  int replicas;                // a power of two, at most 32
   void* ex_x;                  // [n] published (x', dx), tag
   void* ex_y[2];               // [m] published y, tag
   int threads, smem;           // per block

@@ -26,7 +26,7 @@
 // primal step needs them if the step is accepted (a rejected step gathers the old y again).
 // No entry is overwritten while a block may still need it: x'(k + 1) is published after the
 // decision of attempt k, which has every block's sums, posted when its gathers of x'(k) were
-// done; y alternates between two buffers.
+// done; y alternates between two buffers, and so do the posted sums (res_slot).
 // Every wait is bounded as in the cooperative kernel of iter_kernels.cuh.
 //
 // Measured per attempt on a GB300 (three launches -> here): see the table at auto_form() in
@@ -217,20 +217,22 @@ __device__ __forceinline__ void res_warp_sums(T (&v)[N], int step, int used) {
 
 // This block's three sums (of lane 0) posted to every replica under `tag`, and the sums over
 // all blocks in slot order per lane, then a fixed shuffle tree (in lane 0).  Called by one whole warp.
-// (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.)
+// (Replicas: all blocks polling one copy of the slots queued at a few L2 lines.  A second set of
+// slots: a block whose rows need no x' of another block waits for nobody between its decision and
+// its next posting, so it may be an attempt ahead of a block that still reads.)
 // `meanwhile` runs between the posting and the polling.
 template <typename T, typename F>
-__device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* slot, int G,
-                                         unsigned tag, int limit, T (&sum)[3], F meanwhile) {
+__device__ __forceinline__ bool res_sums(DevState* st, typename ResS<T>::Word* slot, int reps,
+                                         int G, unsigned tag, int limit, T (&sum)[3], F meanwhile) {
   using S = ResS<T>;
-  constexpr int reps = res_replicas((int)sizeof(T)), kPoll = sizeof(T) == 8 ? 2 : kResPoll;
+  constexpr int kPoll = sizeof(T) == 8 ? 2 : kResPoll;
   const int lane = threadIdx.x & 31, b = blockIdx.x;
   if constexpr (std::is_same<T, double>::value)
 #pragma unroll
     for (int k = 0; k < 3; ++k) sum[k] = __shfl_sync(0xffffffffu, sum[k], 0);
-  if (lane < reps) S::post(slot + (size_t)lane * G + b, sum, tag);
+  if (lane < reps) S::post(slot + res_slot(tag, reps, lane, G, b), sum, tag);
   meanwhile();
-  const typename S::Word* mine = slot + (size_t)(b % reps) * G;
+  const typename S::Word* mine = slot + res_slot(tag, reps, b & (reps - 1), G, 0);
   bool ok = true;
   sum[0] = sum[1] = sum[2] = (T)0;
   ResWait wait{st, limit, 0};
@@ -703,7 +705,8 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
         if (tid == 0 && att > 0) res_record(&ls, dec);
       };
       if (G > 1)
-        ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, G, tag, wait.limit, s, record) && ok;
+        ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, R.replicas, G, tag, wait.limit, s,
+                         record) && ok;
       else
         record();
       // ---- A6: the same decision in every block

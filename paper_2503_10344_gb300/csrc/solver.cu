@@ -462,9 +462,11 @@ struct ResBufs {
   int *cut_t = nullptr, *cut_a = nullptr;
   ResSizes* sizes = nullptr;
   size_t x_bytes = 0, y_bytes = 0, slot_bytes = 0;
+  int replicas = 0;
   bool ok = false;  // all of them found room
   // `it`: bytes of an iterate element (the words published: resident_kernels.cuh)
-  bool place(const Region* regions, int count, int G, long long m, long long n, int it) {
+  bool place(const Region* regions, int count, int G, long long m, long long n, int it, int reps) {
+    replicas = reps;
     Arena ar[4];
     for (int k = 0; k < count; ++k) ar[k] = Arena{(char*)regions[k].base, 0};
     ok = true;
@@ -482,7 +484,7 @@ struct ResBufs {
     };
     x_bytes = (it == 8 ? 32 : 16) * (size_t)n;
     y_bytes = (it == 8 ? 16 : 8) * (size_t)m;
-    slot_bytes = (it == 8 ? 48 : 16) * (size_t)res_replicas(it) * G;
+    slot_bytes = (it == 8 ? 48 : 16) * (size_t)kResSlotSets * reps * G;
     slot = take(slot_bytes);
     ex_x = take(x_bytes);
     for (void*& y : ex_y) y = take(y_bytes);
@@ -708,7 +710,7 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
       so->res_gv = 1;
       vb = 0;
     }
-    const int G = resident_blocks(mode, nnz);
+    const int G = resident_blocks(mode, nnz), reps = res_replicas(it);  // (half where all do not fit)
     const Region part{bf.part_setup, 8 * setup_part_doubles(m, n)}, tmp{bf.tmp, bf.tmp_bytes};
     if (mode == MODE_FP64) {
       auto upto = [](void* from, void* last, size_t bytes) {  // neighbours in the workspace
@@ -716,9 +718,10 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
       };
       const Region all[4] = {part, upto(bf.stat_r, bf.stat_c, 8 * (size_t)n),
                              upto(bf.tw, bf.sw, 8 * (size_t)m), tmp};
-      so->rb.place(all, 4, G, m, n, it);
-    } else if (!so->rb.place(&part, 1, G, m, n, it)) {
-      so->rb.place(&tmp, 1, G, m, n, it);
+      if (!so->rb.place(all, 4, G, m, n, it, reps)) so->rb.place(all, 4, G, m, n, it, reps / 2);
+    } else if (!so->rb.place(&part, 1, G, m, n, it, reps) && !so->rb.place(&tmp, 1, G, m, n, it, reps) &&
+               !so->rb.place(&part, 1, G, m, n, it, reps / 2)) {
+      so->rb.place(&tmp, 1, G, m, n, it, reps / 2);
     }
     const ResBufs& rb = so->rb;
     if (rb.ok && fits) {
@@ -1265,6 +1268,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     R.cut_t = rb.cut_t;
     R.cut_a = rb.cut_a;
     R.slot = rb.slot;
+    R.replicas = rb.replicas;
     R.ex_x = rb.ex_x;
     R.ex_y[0] = rb.ex_y[0];
     R.ex_y[1] = rb.ex_y[1];

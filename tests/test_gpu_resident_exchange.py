@@ -1,0 +1,35 @@
+"""The exchange of the resident step kernel (persistent_form 4): LPs whose blocks need nothing of one
+another but the sums, so that they run as far apart as the exchange allows.
+
+Tolerances as in test_gpu_resident: a few hundred roundings after 60 fixed steps."""
+import numpy as np
+import pytest
+
+import lpgen
+from test_gpu_resident import F32, F64, FIXED, P, rel  # noqa: F401  (P: the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def uncoupled(pieces, size=8, seed=1):
+    """Independent dense pieces of size x size."""
+    rng = np.random.default_rng(seed)
+    m = pieces * size
+    rows = np.repeat(np.arange(m), size)
+    cols = (rows // size) * size + np.tile(np.arange(size), m)
+    return lpgen._lp(m, m, rows, cols, rng.integers(1, 4, rows.size).astype(float), rng.uniform(0, 2, m),
+                     rng.choice([lpgen.SENSE_GE, lpgen.SENSE_EQ], m), rng.uniform(-1, 1, m),
+                     np.zeros(m), rng.uniform(1, 5, m), np.zeros(m, dtype=np.uint8), f"pieces_{pieces}")
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
+@pytest.mark.parametrize("pieces", [45, 400, 1600])  # a few blocks, about a hundred, every SM
+def test_uncoupled_blocks(P, pieces, prec):  # noqa: F811
+    lp = uncoupled(pieces)
+    tol = F64 if prec == "fp64" else F32
+    x, y, r = P.pdlp_solve(lp, P.default_params(precision=prec, **FIXED))
+    x0, y0, r0 = P.pdlp_solve(lp, P.default_params(precision=prec, lanes_A=2, lanes_AT=2, **FIXED))
+    assert r["persistent_form"] == 4 and r0["persistent_form"] == 0
+    assert rel(x, x0) <= tol and rel(y, y0) <= tol
+    _, _, r = P.pdlp_solve(lp, P.default_params(precision=prec, **dict(FIXED, iter_limit=20000)))
+    assert r["persistent_form"] == 4 and r["iters"] == 20000
