@@ -163,8 +163,11 @@ typedef struct {
                            its iteration or time limit) */
   int debug_skip_barrier; /* fault-handling tests only (default 0): with persistent = 1,
                            block 0 of the persistent step kernel skips its grid-barrier
-                           arrivals, so every block's bounded wait (2^16 polls in this
-                           mode, 2^23 otherwise) runs out; the kernel records the failure
+                           arrivals, and in the form spread over the SMs' shared memory
+                           (persistent_form 4, more than one block) it holds its sums of the
+                           first attempt back until another block has given up, so the
+                           blocks' bounded waits (2^16 polls in this mode, 2^23 otherwise)
+                           run out; the kernel records the failure
                            and returns, and the call returns PDLP_ERR_TIMEOUT with the
                            device context intact */
   int tiles;            /* float32 iterates (PDLP_FP32, PDLP_FP32_BF16A): 1 runs the

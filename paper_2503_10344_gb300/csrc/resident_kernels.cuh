@@ -179,6 +179,12 @@ struct ResWait {
   }
 };
 
+// Fault-handling tests: a block that holds its sums back until another one has given up waiting for
+// them (or for 16 limits).
+__device__ __forceinline__ void res_hold(DevState* st, int limit) {
+  for (int polls = 0; polls < 16 * limit && *(volatile int*)&st->bar_err == 0; ++polls) {}
+}
+
 // n / d for d > 0: the hardware's approximate reciprocal and one residual correction of the
 // quotient (Markstein, "Computation of elementary functions on the IBM RISC System/6000
 // processor", 1990): within an ulp in four instructions.
@@ -634,6 +640,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
   const int ahead_n = nt ? tp[res_chunk_end(tp, nt, R.cap_t, 0)] : 0;  // the first chunk of st
   const ResWait wait{gst, (int)ls.spin_limit, 0};
   ResDecision<T> dec{};
+  const bool hold = b == 0 && G > 1 && ls.bar_skip != 0;
   const long long first_attempt = ls.attempts;
   unsigned ytag = tag0 + 1u;
   bool ahead = false;  // the first chunk of the next primal step is staged
@@ -704,6 +711,7 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
       auto record = [&] {  // of the attempt before, while the sums travel
         if (tid == 0 && att > 0) res_record(&ls, dec);
       };
+      if (hold && att == 0) res_hold(gst, wait.limit);
       if (G > 1)
         ok = res_sums<T>(gst, (typename ResS<T>::Word*)R.slot, R.replicas, G, tag, wait.limit, s,
                          record) && ok;

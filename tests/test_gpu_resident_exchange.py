@@ -33,3 +33,15 @@ def test_uncoupled_blocks(P, pieces, prec):  # noqa: F811
     assert rel(x, x0) <= tol and rel(y, y0) <= tol
     _, _, r = P.pdlp_solve(lp, P.default_params(precision=prec, **dict(FIXED, iter_limit=20000)))
     assert r["persistent_form"] == 4 and r["iters"] == 20000
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
+@pytest.mark.parametrize("name", ["cover", "uncoupled"])
+def test_withheld_sums_time_out_and_the_context_survives(P, name, prec):  # noqa: F811
+    """Block 0 holds its sums back until the others' bounded waits have run out: every block leaves,
+    the call reports PDLP_ERR_TIMEOUT, and the next solve in the same form succeeds."""
+    lp = lpgen.set_cover(7, m=2000, n=8000) if name == "cover" else uncoupled(400)
+    with pytest.raises(P.PdlpError, match="PDLP_ERR_TIMEOUT"):
+        P.pdlp_solve(lp, P.default_params(precision=prec, debug_skip_barrier=1))
+    _, _, r = P.pdlp_solve(lp, P.default_params(precision=prec, iter_limit=200, terminate=0))
+    assert r["persistent_form"] == 4 and r["iters"] == 200
