@@ -129,9 +129,9 @@ struct ResSizes {
 
 struct ResPlan {
   int G;                       // blocks (0: the kernel is not used)
+  int replicas;                // of the posted sums: a power of two, at most 32
   const int *cut_t, *cut_a;    // [G + 1] first column / row of each block
   void* slot;                  // [kResSlotSets][replicas][G] posted sums: ||dx||^2, ||dy||^2, dy^T K dx
-  int replicas;                // a power of two, at most 32
   void* ex_x;                  // [n] published (x', dx), tag
   void* ex_y[2];               // [m] published y, tag
   int threads, smem;           // per block
