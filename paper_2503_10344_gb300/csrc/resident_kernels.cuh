@@ -753,7 +753,13 @@ __global__ void __launch_bounds__(kResBlock, 1) k_resident(IterData<T, V> d, Res
     d.y[cur][a0 + i] = ys[cur][i];
     d.sum_y[a0 + i] = sy[i];
   }
-  if (b == 0 && tid == 0) store_step_state(gst, ls);
+  if (b == 0 && tid == 0) {
+    store_step_state(gst, ls);
+    // others may have given up on this block's last sums and left without their part of the
+    // iterate (they flag bar_err before the status, which was overwritten just now)
+    __threadfence();
+    if (*(volatile int*)&gst->bar_err != 0) atomicExch(&gst->status, kStatusWaitFailed);
+  }
 }
 
 }  // namespace pdlp

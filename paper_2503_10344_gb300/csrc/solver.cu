@@ -1572,7 +1572,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     ms_solve = (float)(1e3 * std::chrono::duration<double>(h2 - h1).count());
   }
 
-  if (fs.status == kStatusWaitFailed)
+  if (fs.status == kStatusWaitFailed || fs.bar_err)
     return fail(PDLP_ERR_TIMEOUT,
                 "a bounded wait of a step kernel gave up (a grid barrier of the persistent kernel "
                 "or a staged copy of the tile kernels)");

@@ -45,3 +45,17 @@ def test_withheld_sums_time_out_and_the_context_survives(P, name, prec):  # noqa
         P.pdlp_solve(lp, P.default_params(precision=prec, debug_skip_barrier=1))
     _, _, r = P.pdlp_solve(lp, P.default_params(precision=prec, iter_limit=200, terminate=0))
     assert r["persistent_form"] == 4 and r["iters"] == 200
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_late_sums_of_the_last_attempt_still_fail_the_solve(P, prec):  # noqa: F811
+    """With one attempt per check period block 0's late sums complete its own attempt: it leaves as
+    after a success, while the others have left without their part of the iterate."""
+    lp = lpgen.set_cover(7, m=2000, n=8000)
+    kw = dict(precision=prec, adaptive_step=0, check_period=1)
+    with pytest.raises(P.PdlpError, match="PDLP_ERR_TIMEOUT"):
+        P.pdlp_solve(lp, P.default_params(debug_skip_barrier=1, iter_limit=50, **kw))
+    with pytest.raises(P.PdlpError, match="PDLP_ERR_TIMEOUT"):
+        P.pdlp_solve(lp, P.default_params(debug_skip_barrier=1, iter_limit=1, **kw))
+    _, _, r = P.pdlp_solve(lp, P.default_params(iter_limit=50, terminate=0, **kw))
+    assert r["persistent_form"] == 4 and r["iters"] == 50
