@@ -781,6 +781,7 @@ struct GraphEntry {
   cudaGraphExec_t exec;
   long long nodes;
   unsigned long long used;
+  int users;  // solves that hold it now: only an entry without any is evicted
 };
 static std::mutex g_graph_mu;
 static std::vector<GraphEntry>* g_graphs = new std::vector<GraphEntry>();
@@ -802,6 +803,55 @@ static GraphKey graph_key(const Solve& sv, int period) {
   memcpy(&k.kr, &sv.kr, sizeof(KktRaw));
   return k;
 }
+
+// A solve's hold on its graph: on a cache entry, or on a graph of its own where every entry of the
+// full cache is held by another thread's solve.  Given up when its launches are done.
+struct GraphHold {
+  cudaStream_t s;
+  cudaGraphExec_t exec = nullptr;
+  long long nodes = 0;
+  bool cached = false, idle = false;
+  explicit GraphHold(cudaStream_t stream) : s(stream) {}
+  GraphHold(const GraphHold&) = delete;
+  bool find(const GraphKey& key) {
+    std::lock_guard<std::mutex> lk(g_graph_mu);
+    for (GraphEntry& e : *g_graphs)
+      if (e.key == key) {
+        e.used = ++g_graph_clock;
+        ++e.users;
+        exec = e.exec;
+        nodes = e.nodes;
+        return cached = true;
+      }
+    return false;
+  }
+  void add(const GraphKey& key, cudaGraphExec_t graph, long long count) {
+    exec = graph;
+    nodes = count;
+    std::lock_guard<std::mutex> lk(g_graph_mu);
+    if (g_graphs->size() >= kGraphCacheSize) {
+      auto old = g_graphs->end();
+      for (auto e = g_graphs->begin(); e != g_graphs->end(); ++e)
+        if (e->users == 0 && (old == g_graphs->end() || e->used < old->used)) old = e;
+      if (old == g_graphs->end()) return;
+      cudaGraphExecDestroy(old->exec);
+      g_graphs->erase(old);
+    }
+    g_graphs->push_back(GraphEntry{key, exec, nodes, ++g_graph_clock, 1});
+    cached = true;
+  }
+  ~GraphHold() {
+    if (!exec) return;
+    if (!idle) cudaStreamSynchronize(s);
+    if (!cached) {
+      cudaGraphExecDestroy(exec);
+      return;
+    }
+    std::lock_guard<std::mutex> lk(g_graph_mu);
+    for (GraphEntry& e : *g_graphs)
+      if (e.exec == exec) --e.users;
+  }
+};
 
 // ---------------------------------------------------------------- pinned mirrors
 // The pinned host copy of the state that a solve polls.  Allocating and freeing one per solve
@@ -1408,22 +1458,9 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
       cudaEventDestroy(e[1]);
     }
   } ev2{ev};
-  cudaGraphExec_t gexec = nullptr;
-  long long graph_nodes = 0;
-  bool cached = false;
+  GraphHold hold(s);
   const GraphKey gkey = graph_key(sv, p->check_period);
-  if (p->iter_limit > 0) {
-    std::lock_guard<std::mutex> lk(g_graph_mu);
-    for (GraphEntry& e : *g_graphs)
-      if (e.key == gkey) {
-        gexec = e.exec;
-        graph_nodes = e.nodes;
-        e.used = ++g_graph_clock;
-        cached = true;
-        break;
-      }
-  }
-  if (p->iter_limit > 0 && !cached) {
+  if (p->iter_limit > 0 && !hold.find(gkey)) {
     cudaStream_t cs;
     CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     struct SFree {
@@ -1498,19 +1535,13 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
       CUDA_TRY(ee);
       gd.keep = true;
     }
-    graph_nodes = g_launches - before;
+    const long long nodes = g_launches - before;
     g_launches = before;
+    cudaGraphExec_t gexec = nullptr;
     cudaError_t ie = cudaGraphInstantiate(&gexec, graph, 0);
     cudaGraphDestroy(graph);
     CUDA_TRY(ie);
-    std::lock_guard<std::mutex> lk(g_graph_mu);
-    if (g_graphs->size() >= kGraphCacheSize) {
-      auto old = std::min_element(g_graphs->begin(), g_graphs->end(),
-                                  [](const GraphEntry& a, const GraphEntry& b) { return a.used < b.used; });
-      cudaGraphExecDestroy(old->exec);
-      g_graphs->erase(old);
-    }
-    g_graphs->push_back(GraphEntry{gkey, gexec, graph_nodes, ++g_graph_clock});
+    hold.add(gkey, gexec, nodes);
   }
   phase("graph capture + instantiate");
 
@@ -1520,9 +1551,9 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
   const long long max_launches =
       (p->iter_limit / p->check_period + 2) * 64 + 1024;  // rejections re-run a chunk
   auto launch = [&]() -> cudaError_t {
-    cudaError_t e = cudaGraphLaunch(gexec, s);
+    cudaError_t e = cudaGraphLaunch(hold.exec, s);
     if (e != cudaSuccess) return e;
-    g_launches += graph_nodes;
+    g_launches += hold.nodes;
     e = cudaMemcpyAsync(&hm[launched & 1], bf.st, 16, cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return e;
     e = cudaEventRecord(ev[launched & 1], s);
@@ -1551,7 +1582,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     }
   }
   CUDA_TRY(cudaStreamSynchronize(s));  // drain the chunk launched behind the terminating one
-  pinned.idle = true;
+  pinned.idle = hold.idle = true;
   phase("iterations");
   CUDA_TRY(cudaEventRecord(e2, s));
   }  // graph-driven iteration phase
