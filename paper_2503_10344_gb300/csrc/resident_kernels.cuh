@@ -185,10 +185,19 @@ __device__ __forceinline__ void res_hold(DevState* st, int limit) {
   for (int polls = 0; polls < 16 * limit && *(volatile int*)&st->bar_err == 0; ++polls) {}
 }
 
-// n / d for d > 0: the hardware's approximate reciprocal and one residual correction of the
-// quotient (Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990): within an ulp in four instructions.
+// n / d for n >= 0, d > 0 without the division's branch to its rare cases: the hardware's approximate
+// reciprocal r and one residual correction of the quotient (Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990).  r is within an ulp, so n r is within
+// 1.5 2^-23 of the quotient; the residual is exact but for its last bit, and what is left before the
+// final rounding is of relative size 2^-45: an error of (1/2 + 2^-20) ulp, where n is above 2^-90
+// (below, that of n as the square of a float32 number is larger).  A d whose reciprocal is no normal
+// number (0 / d would be 0 times infinity) is first scaled, with n, by a power of two.
+// n / d itself in the loops over the rows: 0.35 us more per attempt (covering LP of 2,000 rows
+// 4.3 -> 4.6, 10,000 rows 5.4 -> 5.7, 50,000 rows 12.6 -> 13.1, 200 x 400 relaxation 2.2 -> 2.55).
 __device__ __forceinline__ float div_pos(float n, float d) {
+  const float s = d < 0x1p-100f ? 0x1p64f : d > 0x1p100f ? 0x1p-64f : 1.0f;
+  n *= s;
+  d *= s;
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
   const float q = n * r;
