@@ -778,23 +778,29 @@ __global__ void __launch_bounds__(NB) k_gnn_head(int N, const float* __restrict_
 struct Seg {
   int src, len, dst;
 };
-// a += x with the rounding error kept in e (Knuth's two-sum): float32 additions that together carry
-// twice the digits
-__device__ __forceinline__ void two_sum(float& a, float& e, float x) {
-  const float s = a + x, b = s - a;
-  e += (a - (s - b)) + (x - b);
+// a += x; what the rounding cut off (Knuth's two-sum)
+__device__ __forceinline__ float two_sum(float& a, float x) {
+  const float s = a + x, b = s - a, cut = (a - (s - b)) + (x - b);
   a = s;
+  return cut;
 }
+// a sum as three float32 numbers: what is cut off from the first goes to the second, from that to
+// the third, so that its error is below that of a float64 sum
+struct Sum3 {
+  float a, b, c;
+  __device__ __forceinline__ void add(float x) { c += two_sum(b, two_sum(a, x)); }
+};
 // grad[dst + e] += scale * sum_b part[b * stride + src + e].  A block takes 32 elements: 32 warps
 // each add every 32nd partial of them (one 128-byte line per warp and partial), then one warp adds
-// the 32 sums in order.  The sums are pairs of float32 numbers (an error of 2^-46, as good as the
-// float64 sums that they replace, whose conversions and additions held the float64 pipe: 2.5
-// million of each for the 304 partials of a dense layer; 15.0 -> 8.0 us on average).
+// the 32 sums in order.  In float64 the conversions and additions held that pipe (2.5 million of
+// each for the 304 partials of a dense layer); the float32 triples cost thirteen additions of the
+// other pipe and are no less accurate.  A sum that leaves their range (or is undefined) is added up
+// again in float64.
 constexpr int kReduceNB = 1024;
 __global__ void __launch_bounds__(kReduceNB) k_gnn_reduce(const float* __restrict__ part, int nblk,
                                                           int stride, Seg s0, Seg s1, Seg s2,
                                                           float* __restrict__ grad, float scale) {
-  __shared__ float2 sh[kReduceNB / 32][32];
+  __shared__ Sum3 sh[kReduceNB / 32][32];
   const int total = s0.len + s1.len + s2.len, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
   Seg s = s0;
@@ -807,21 +813,27 @@ __global__ void __launch_bounds__(kReduceNB) k_gnn_reduce(const float* __restric
       s = s2;
     }
   }
-  float acc = 0.f, err = 0.f;
+  const float* p = part + s.src + i;
+  Sum3 sum{0.f, 0.f, 0.f};
   if (e < total) {
-    const float* p = part + s.src + i;
 #pragma unroll 10
-    for (int b = w; b < nblk; b += kReduceNB / 32) two_sum(acc, err, p[(size_t)b * stride]);
+    for (int b = w; b < nblk; b += kReduceNB / 32) sum.add(p[(size_t)b * stride]);
   }
-  sh[w][lane] = make_float2(acc, err);
+  sh[w][lane] = sum;
   __syncthreads();
   if (w == 0 && e < total) {
     for (int k = 1; k < kReduceNB / 32; ++k) {
-      const float2 v = sh[k][lane];
-      two_sum(acc, err, v.x);
-      err += v.y;
+      const Sum3 v = sh[k][lane];
+      sum.add(v.a);
+      sum.add(v.b);
+      sum.c += v.c;
     }
-    grad[s.dst + i] += scale * (isfinite(acc) ? acc + err : acc);
+    double all = (double)sum.a + ((double)sum.b + (double)sum.c);
+    if (!isfinite(all)) {
+      all = 0.0;
+      for (int b = 0; b < nblk; ++b) all += (double)p[(size_t)b * stride];
+    }
+    grad[s.dst + i] += scale * (float)all;
   }
 }
 

@@ -36,3 +36,36 @@ def test_dense_layers_at_tile_edges(P, m, n):  # noqa: F811
     ycanon = np.where(lp.sense == ord("L"), -ys, ys)
     _, want = G.grad(theta.astype(np.float64), G.graph(lp), xs, ycanon)
     assert rel(md.grad(), want) <= TOL, rel(md.grad(), want)
+
+
+def test_gradient_sums_beyond_the_range_of_float32(P):  # noqa: F811
+    """Labels of 3e36 in the first half of the rows and -3e36 in the second: the partial sums of a
+    head weight's gradient leave the range of float32 on the way to a sum within it.  (TOL of the sum
+    of the terms' magnitudes.)"""
+    n = 4096
+    lp = lpgen.random_sparse_lp(3, 64, n, density=0.02)
+    lp.l[:], lp.u[:] = 0.0, np.inf
+    theta = biased_params(5)
+    d = G.unpack(theta.astype(np.float64))
+    for name, _ in G.param_shapes():
+        if name.startswith("b"):
+            d[name] *= 8.0
+    theta = G.pack(d).astype(np.float32)
+    xs, ys = labels(lp, 1)
+    xs = np.where(np.arange(n) < n // 2, 3e36, -3e36)
+    md = P.GnnModel(seed=0)
+    md.set_params(theta)
+    g = md.graph(lp, xs, ys)
+    md.zero_grad()
+    md.backward(g, scale=1.0)
+    graph = G.graph(lp)
+    h = G.forward(theta.astype(np.float64), graph, keep=True)[2]["hv"][-1]
+    ycanon = np.where(lp.sense == ord("L"), -ys, ys)
+    _, want = G.grad(theta.astype(np.float64), graph, xs, ycanon)
+    got = G.unpack(md.grad().astype(np.float64))["w_x"]
+    want = G.unpack(want)["w_x"]
+    terms = 3e36 * 2.0 / n * h.sum(axis=0)
+    top = float(np.finfo(np.float32).max)
+    assert np.max(0.5 * terms) > 1.1 * top and np.max(np.abs(want)) < 0.9 * top
+    assert np.all(np.isfinite(got))
+    assert np.all(np.abs(got - want) <= TOL * terms)
