@@ -508,7 +508,9 @@ __global__ void __launch_bounds__(NB, 2) k_gnn_dense(int N, const float* __restr
 // per-block partials of X1^T dP, X2^T dP (row-major [in][out]) and sum_r dP.
 // A block stages the pieces of 64 rows of [X1 | X2] and dP in shared memory; four warps form dX1
 // of the rows, four dX2 (16 rows each), then each warp its 16 of the 128 rows of the weight
-// gradients, where both operands are in pieces: the six products above 2^-24.
+// gradients, where both operands are in pieces: all nine products.  (Without the smallest three, of
+// the sign of their terms, weight gradients were cut by 2.6e-8 towards zero on average; they cost 48 us
+// of 2,580 in the gradient of four graphs of 12,500 x 50,000.)
 // The rows of shared memory are padded to an odd number of 16-byte units (ldmatrix).
 constexpr int kXStride = 136, kBwdRows = 64;
 constexpr int kBwdSmem = (3 * kBwdRows * (kXStride + kDStride) + 128 * kDStride) * 2;
@@ -625,6 +627,9 @@ __global__ void __launch_bounds__(NB, 2) k_gnn_dense_bwd(int N, const float* __r
             mma16(r, a[1], b[1][2 * k], b[1][2 * k + 1]);
             mma16(r, a[2], b[0][2 * k], b[0][2 * k + 1]);
             mma16(r, a[0], b[2][2 * k], b[2][2 * k + 1]);
+            mma16(r, a[2], b[1][2 * k], b[1][2 * k + 1]);
+            mma16(r, a[1], b[2][2 * k], b[2][2 * k + 1]);
+            mma16(r, a[2], b[2][2 * k], b[2][2 * k + 1]);
           });
         }
       }

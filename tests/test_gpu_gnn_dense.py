@@ -69,3 +69,27 @@ def test_gradient_sums_beyond_the_range_of_float32(P):  # noqa: F811
     assert np.max(0.5 * terms) > 1.1 * top and np.max(np.abs(want)) < 0.9 * top
     assert np.all(np.isfinite(got))
     assert np.all(np.abs(got - want) <= TOL * terms)
+
+
+def test_weight_gradients_are_not_cut_towards_zero(P):  # noqa: F811
+    """Both operands of a weight gradient are truncated into pieces, so a product of small pieces that
+    is left out has the sign of its term: with terms of one sign (labels far below the predictions)
+    the smallest three products are 2^-24 of the sum on average.  Exact products leave no such bias:
+    under a quarter of that, over the layers' weights of four graphs."""
+    cut = []
+    for seed in range(1, 5):
+        lp = lpgen.set_cover(seed, m=3000, n=12000)
+        rng = np.random.default_rng(seed)
+        xs, ys = rng.random(lp.n) - 5.0, rng.random(lp.m) + 5.0 * float(np.max(np.abs(lp.c)))
+        theta = biased_params(seed)
+        md = P.GnnModel(seed=0)
+        md.set_params(theta)
+        g = md.graph(lp, xs, ys)
+        md.zero_grad()
+        md.backward(g, scale=1.0)
+        _, want = G.grad(theta.astype(np.float64), G.graph(lp), xs, ys)
+        got, want = G.unpack(md.grad().astype(np.float64)), G.unpack(want)
+        for k in want:
+            if k.startswith("W_") and k[-1].isdigit():
+                cut.append(np.sum((got[k] - want[k]) * np.sign(want[k])) / np.sum(np.abs(want[k])))
+    assert np.mean(cut) > -0.25 * 2.0 ** -24, np.mean(cut)
