@@ -252,8 +252,9 @@ typedef struct {
                              vectors and iterates fit: 76 KB for a 200 x 400 relaxation
                              with 1,600 nonzeros in float64), 4 the LP spread over the
                              shared memory of all SMs (chosen with persistent = 0 where
-                             it fits; float64 solves that record iterates or the decision
-                             trace run as form 0) */
+                             it fits; float64 solves that record iterates without the
+                             decision trace run as form 0: such iterates agree with those of
+                             the plain solve to rounding, not bit for bit) */
   double spectral_norm;   /* halpern = 1: L, the power-iteration estimate of ||K~||_2 the
                              step size came from; 0 otherwise */
 } pdlp_result;

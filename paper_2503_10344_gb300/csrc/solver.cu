@@ -562,11 +562,16 @@ struct SetupOut {
 constexpr int kResNnz = 512, kResNnz64 = 256;
 constexpr int kOneBlockNnz = 2500, kOneBlockNnz64 = 1000;
 static int one_block_nnz(Mode mode) { return mode == MODE_FP64 ? kOneBlockNnz64 : kOneBlockNnz; }
-// Float64 solves that record iterates or decisions are parity runs against a reference: they keep
-// the separate launches, whose order of summation such records were made with.
+static bool records_decisions(const pdlp_diagnostics* dg) {
+  return dg && dg->attempt_capacity > 0 && dg->eta && dg->eta_bar && dg->accepted;
+}
+// Float64 solves that record the iterates alone are parity runs against a reference: they keep the
+// separate launches, whose order of summation such records were made with.  A decision trace is that
+// of the run itself, with whatever is recorded beside it: under the adaptive rule two orders of
+// summation part, tenfold every 40 steps.
 static bool parity_run(Mode mode, const pdlp_diagnostics* dg) {
-  return mode == MODE_FP64 && dg &&
-         (dg->x_cur || dg->y_cur || dg->x_avg || dg->y_avg || dg->attempt_capacity > 0);
+  return mode == MODE_FP64 && dg && !records_decisions(dg) &&
+         (dg->x_cur || dg->y_cur || dg->x_avg || dg->y_avg);
 }
 static bool auto_form(const pdlp_params* p, int m, long long nnz) {
   return p->persistent == 0 && !p->tiles && !p->halpern && !p->autotune && !p->lanes_A &&
@@ -1265,7 +1270,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     hs.fac_inc_f = bf.fac->inc_f;
     hs.fac_n = kFacN;
   }
-  if (dg && dg->attempt_capacity > 0 && dg->eta && dg->eta_bar && dg->accepted) {
+  if (records_decisions(dg)) {
     hs.tr_eta = dg->eta;
     hs.tr_eta_bar = dg->eta_bar;
     hs.tr_accepted = (signed char*)dg->accepted;
