@@ -538,30 +538,44 @@ struct SetupOut {
 // lanes, tiles, the autotuner or the Halpern variant): the LP in one block's shared memory up to
 // one_block_nnz() nonzeros; spread over the SMs' shared memory
 // (resident_kernels.cuh) while it fits there, else three launches per attempt.  Measured per
-// attempt on a GB300 (us; values in float32 / bfloat16 or the 0/1 pattern):
+// attempt with a fixed step on a GB300 (us; values in float32 / bfloat16 or the 0/1 pattern):
 //                                 nonzeros   three launches   one block     resident
-//   relaxation 200 x 400             1,670      9.9 /  9.4    2.1 /  2.2    3.5 /  3.3
-//   relaxation 400 x 800             3,238     10.0 /  9.6    2.8           3.5
-//   relaxation 2,000 x 4,000        15,963     13.4 / 12.0   30.3 / 36.4          3.8
-//   covering 2,000 x 8,000          54,130     12.4 / 11.6                        4.1
-//   covering 10,000 x 40,000       269,989     14.2 / 13.0                        5.6
-//   covering 50,000 x 200,000    1,350,409     23.0 / 20.5                 20.3 / 12.8
-//   energy system, 24 h             21,600     23.3                         4.4
-//   energy system, 720 h           648,000     17.7                         9.9
+//   relaxation 200 x 400             1,606      9.9 /  9.4    2.1 /  2.3    3.5 /  3.3
+//   covering 100 x 400               2,668                    2.3 /  2.1    3.8 /  3.8
+//   relaxation 400 x 800             3,139     10.0 /  9.6    2.8 /  3.1    3.6 /  3.6
+//   relaxation 300 x 600             3,642                    3.2 /  3.6    3.9 /  3.9
+//   relaxation 500 x 1,000           4,005                    3.5 /  3.9    3.8 /  3.8
+//   relaxation 600 x 1,200           4,843                    3.9 /  4.4    3.6 /  3.6
+//   relaxation 2,000 x 4,000        15,963     13.4 / 10.5   30.3 / 36.4          4.0
+//   covering 2,000 x 8,000          54,130     12.4 / 12.1                        4.4
+//   covering 10,000 x 40,000       269,989     14.2 / 13.3                        5.4
+//   covering 50,000 x 200,000    1,350,409     22.3 / 20.3                 18.5 / 12.5
+//   energy system, 24 h             21,600     21.1                         4.5
+//   energy system, 720 h           648,000     18.8                  9.9 to 11.6
 // and in float64 (the one block's chains of float64 operations are about as long as the exchange):
 //   relaxation 40 x 80                 320     15.5             4.1           5.0
-//   relaxation 200 x 400             1,670     16.6             6.6           6.6
-//   relaxation 2,000 x 4,000        15,963     19.1                           7.6
-//   covering 2,000 x 8,000          54,130     25.8                           9.0
-//   covering 10,000 x 40,000       269,989     33.7                          13.2
-//   covering 25,000 x 100,000      675,211     40.0                          25.7
-//   energy system, 24 h             21,600     23.7                          10.0
+//   covering 40 x 160                1,087                      5.2           6.0
+//   relaxation 200 x 400             1,606     19.3             6.6           6.3
+//   relaxation 2,000 x 4,000        15,963     21.8                           7.6
+//   covering 2,000 x 8,000          54,130     26.0                           9.1
+//   covering 10,000 x 40,000       269,989     32.8                          13.2
+//   covering 25,000 x 100,000      675,211     39.6                          25.6
+//   energy system, 24 h             21,600     26.1                           9.8
 //   energy system, 400 h           360,000    129.0                          17.6
+// The adaptive rule (the default) adds to the one block and the resident kernel 0.0-0.1 us in
+// float32 and 1.1-1.3 us in float64 (its divisions are on the way from one attempt to the next), to
+// the launches nothing.
 // kResNnz nonzeros per block: 256 and 1,024 measured within 10 % of 512, slower on most; in
 // float64 256 (128: 3-6 % slower, 512: 2 % faster to 10 % slower).
+// The line between the first two lies at the sizes above for rows and columns of up to
+// kOneBlockAvg entries on average; at most eight lanes walk a row there, so with longer ones it stays
+// lower.
 constexpr int kResNnz = 512, kResNnz64 = 256;
-constexpr int kOneBlockNnz = 2500, kOneBlockNnz64 = 1000;
-static int one_block_nnz(Mode mode) { return mode == MODE_FP64 ? kOneBlockNnz64 : kOneBlockNnz; }
+constexpr int kOneBlockNnz = 2500, kOneBlockNnzShort = 3700, kOneBlockAvg = 32, kOneBlockNnz64 = 1000;
+static int one_block_nnz(Mode mode, long long m, long long n, long long nnz) {
+  if (mode == MODE_FP64) return kOneBlockNnz64;
+  return nnz <= kOneBlockAvg * std::min(m, n) ? kOneBlockNnzShort : kOneBlockNnz;
+}
 static bool records_decisions(const pdlp_diagnostics* dg) {
   return dg && dg->attempt_capacity > 0 && dg->eta && dg->eta_bar && dg->accepted;
 }
@@ -586,6 +600,13 @@ static int optin_smem() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   return optin;
+}
+// a small LP whose form is ours to choose and that fits in one block's shared memory
+static bool one_block(const pdlp_params* p, Mode mode, long long m, long long n, long long nnz,
+                      const pdlp_diagnostics* dg) {
+  return auto_form(p, (int)m, nnz) && nnz <= one_block_nnz(mode, m, n, nnz) && !parity_run(mode, dg) &&
+         smem_layout(m, n, nnz, mode == MODE_FP64 ? 8 : 4, mode != MODE_PAT,
+                     mode == MODE_BF16 || mode == MODE_PAT).bytes <= optin_smem() - kSmemStatic;
 }
 
 // Validation, canonical form, transpose, value format, scaling, iteration-space
@@ -701,7 +722,8 @@ static int setup_lp(const pdlp_csr* A, const double* b, const char* sense, const
   so->res_G = so->res_gv = 0;
   so->rb = ResBufs{};
   so->res = ResSizes{};
-  if (auto_form(p, m, nnz) && nnz > one_block_nnz(mode) && !parity_run(mode, dg)) {
+  if (auto_form(p, m, nnz) && nnz > (mode == MODE_FP64 ? kOneBlockNnz64 : kOneBlockNnz) &&
+      !parity_run(mode, dg) && !one_block(p, mode, m, n, nnz, dg)) {
     const int it = mode == MODE_FP64 ? 8 : 4;
     int vb = mode == MODE_FP64 ? 8 : mode == MODE_FP32 ? 4 : mode == MODE_BF16 ? 2 : 0;
     const long long data = nnz * 2 * (4 + vb) + 6LL * it * ((long long)m + n);
@@ -1371,10 +1393,7 @@ static int solve_device(const pdlp_csr* A, const double* b, const char* sense, c
     }
   }
   // one block: asked for, or a small LP whose form is ours to choose (and which fits: below)
-  const bool small = auto_form(p, m, nnz) && nnz <= one_block_nnz(mode) && !parity_run(mode, dg) &&
-                     smem_layout(m, n, nnz, mode == MODE_FP64 ? 8 : 4, mode != MODE_PAT,
-                                 mode == MODE_BF16 || mode == MODE_PAT).bytes <=
-                         optin_smem() - kSmemStatic;
+  const bool small = one_block(p, mode, m, n, nnz, dg);
   if (p->persistent || small) {
     // the resident grid of the persistent kernel (probe launch with nothing to do:
     // the state says check_due, so every block returns at entry)

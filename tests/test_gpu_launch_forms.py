@@ -51,3 +51,14 @@ def test_launches_reach_the_tolerance(P, name, lanes, prec):  # noqa: F811
     assert r["status"] == P.PDLP_OPTIMAL and r["persistent_form"] == 0
     assert (r["lanes_A"], r["lanes_AT"]) == lanes
     assert O.kkt_original(lp, x, y).rel_kkt <= 1.01e-4
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_one_block_up_to_where_it_is_faster(P, prec):  # noqa: F811
+    def form(lp):
+        return P.pdlp_solve(lp, P.default_params(iter_limit=5, terminate=0, precision=prec))[2]["persistent_form"]
+
+    assert form(lpgen.set_cover(1, m=100, n=400)) == 3                              # 2,668 nonzeros
+    assert form(lpgen.mip_relaxation(1, m=300, n=600)) == 3                         # 3,642
+    assert form(lpgen.mip_relaxation(1, m=600, n=1200, density=4 / 600)) == 4       # 4,843
+    assert form(lpgen.random_sparse_lp(1, 20, 1500, density=0.1)) == 4              # 3,000, long rows

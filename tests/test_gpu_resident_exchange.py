@@ -23,7 +23,7 @@ def uncoupled(pieces, size=8, seed=1):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
-@pytest.mark.parametrize("pieces", [45, 400, 1600])  # a few blocks, about a hundred, every SM
+@pytest.mark.parametrize("pieces", [60, 400, 1600])  # a few blocks, about a hundred, every SM
 def test_uncoupled_blocks(P, pieces, prec):  # noqa: F811
     lp = uncoupled(pieces)
     tol = F64 if prec == "fp64" else F32
