@@ -1520,7 +1520,7 @@ __global__ void k_batch_ingest(const BatchLp* lps, int64_t* rp_g, int* col_g, do
 }
 
 // The A3 scalars of each LP, as k_iter_vectors and k_absmax_scaled take them for one LP:
-// gridDim.x blocks per LP each leave 7 sums and the bits of a maximum in part[], and one warp
+// gridDim.x blocks per LP each leave 7 sums and the bits of a maximum in part[], and one thread
 // per LP adds them up in order (one block per LP walked 555,000 nonzeros alone and left most
 // of the chip idle: 5.86 -> 0.44 ms for 96 covering sub-LPs).
 __global__ void __launch_bounds__(kBlock) k_batch_scalars(const BatchLp* lps, const double* dr,
