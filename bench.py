@@ -173,6 +173,15 @@ def ncu_traffic(kernel: str, precision: str, workload: str = "set_cover"):
     return None
 
 
+def dominant_kernel(kt: dict) -> str:
+    """The kernel that a solve spends its steps in, of the timings of P.time_kernels: the one that
+    holds a whole check period, where the solve's form has one (its primal and dual kernels are
+    timed all the same, but not launched), else the longer of the two half-steps."""
+    if kt["persistent_attempt"]["ms"] > 0:
+        return "persistent_attempt"
+    return max(("primal_step", "dual_step"), key=lambda k: kt[k]["ms"])
+
+
 # ------------------------------------------------------------------ CPU oracle
 CPU_SNIPPET = r"""
 import json, sys, time
@@ -389,14 +398,12 @@ def run_gpu(args):
     peaks = _j.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else None
     peak = peaks["hbm_gbs"] if peaks else 6800.0
-    # the persistent kernel (persistent = 1, not the default) runs every step attempt of a
-    # check period in one launch; the two-launch form times its primal and dual kernels apart
-    if prm.persistent and kt["persistent_attempt"]["ms"] > 0:
-        dom = "persistent_attempt"
-    else:
-        dom = max(("primal_step", "dual_step"), key=lambda k: kt[k]["ms"])
+    dom = dominant_kernel(kt)
     ach = kt[dom]["bytes"] / (kt[dom]["ms"] * 1e-3) / 1e9
-    roof = {"bound": "hbm", "kernel": dom, "achieved": ach, "peak": peak, "unit": "GB/s",
+    # (forms 3 and 4 hold the LP's step data in shared memory: the bytes are those of an attempt
+    # that streams them, and what it waits for is gathers through L2)
+    roof = {"bound": "hbm" if res["persistent_form"] in (0, 1, 2) else "on chip", "kernel": dom,
+            "persistent_form": res["persistent_form"], "achieved": ach, "peak": peak, "unit": "GB/s",
             "frac": ach / peak, "traffic": ncu_traffic(dom, args.precision),
             "peak_source": "measured" if peaks else "fallback",
             "kernels": {k: {"us": 1e3 * v["ms"], "bytes": v["bytes"],
@@ -628,9 +635,9 @@ def c5_section(args, dev, stream, peak, train=160, test=20, mmin=5_000, mmax=20_
 
 def c1_section(args, dev, stream, peak):
     """The 200 x 400 MIP relaxation (seeds 1..20): float64 PDLP to rel. KKT 1e-4 and to
-    1e-8 through the host API (latency of a small LP: setup, iterations, copies), with
-    the two-launch step kernels and with the one-block persistent kernel
-    (persistent = 2), then fix-and-propagate (Frac order) from the 1e-4 point with its
+    1e-8 through the host API (latency of a small LP: setup, iterations, copies), in the
+    form that the library chooses (persistent = 0) and with the one-block persistent
+    kernel (persistent = 2), then fix-and-propagate (Frac order) from the 1e-4 point with its
     final LP at 1e-8."""
     import lpgen
     import paper_2503_10344_gb300 as P
@@ -651,6 +658,7 @@ def c1_section(args, dev, stream, peak):
             rows.append(row)
         med = lambda key, tol: float(np.median([r[tol][key] for r in rows]))
         out[f"persistent{persistent}"] = {
+            "persistent_form": r["persistent_form"],
             "time_to_1e-4_s": {"median_wall": med("wall_s", 1e-4), "median_solve": med("solve_s", 1e-4)},
             "time_to_1e-8_s": {"median_wall": med("wall_s", 1e-8), "median_solve": med("solve_s", 1e-8)},
             "iters_1e-4_median": med("iters", 1e-4), "iters_1e-8_median": med("iters", 1e-8),
