@@ -430,13 +430,13 @@ def run_gpu(args):
                 extra[key] = {"error": str(e)[:300]}
         if not args.no_cpu_baseline:
             # the oracle beside the two workloads that stream from HBM, on bounded samples
-            for key, maker, iters, what in (
+            for key, maker, sample, what in (
                     ("energy", "[lpgen.energy_system()]", 16, "the energy system"),
                     ("batch", "lpgen.set_cover_batch(count=8)", 64,
                      "each of the first 8 sub-LPs of the batch")):
                 if key in extra and "error" not in extra[key]:
                     try:
-                        extra[key]["cpu_baseline"] = cpu_oracle_workload(maker, iters, what)
+                        extra[key]["cpu_baseline"] = cpu_oracle_workload(maker, sample, what)
                     except Exception as e:
                         extra[key]["cpu_baseline"] = {"error": str(e)[:200]}
     if rank == 0:
