@@ -164,8 +164,8 @@ typedef struct {
   int debug_skip_barrier; /* fault-handling tests only (default 0): with persistent = 1,
                            block 0 of the persistent step kernel skips its grid-barrier
                            arrivals, and in the form spread over the SMs' shared memory
-                           (persistent_form 4, more than one block) it holds its sums of the
-                           first attempt back until another block has given up, so the
+                           (persistent_form 4, more than one block) it begins its first
+                           attempt only when another block has given up, so the
                            blocks' bounded waits (2^16 polls in this mode, 2^23 otherwise)
                            run out; the kernel records the failure
                            and returns, and the call returns PDLP_ERR_TIMEOUT with the

@@ -101,7 +101,7 @@ struct DevState {
   unsigned int bar_count, bar_gen;
   int bar_err;
   int bar_skip;          // fault-handling tests: block 0 skips its barrier arrivals, or (resident
-                         // kernel) posts its sums only when another block has given up
+                         // kernel) begins only when another block has given up
   long long spin_limit;  // polls of one barrier wait before it gives up
   // reflected restarted Halpern PDHG (halpern = 1; pdlp_params.halpern): a step maps the
   // Halpern iterate z through the PDHG operator T and mixes z' = ha T(z) + hb z + hc z_a

@@ -38,8 +38,9 @@ def test_uncoupled_blocks(P, pieces, prec):  # noqa: F811
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
 @pytest.mark.parametrize("name", ["cover", "uncoupled"])
 def test_withheld_sums_time_out_and_the_context_survives(P, name, prec):  # noqa: F811
-    """Block 0 holds its sums back until the others' bounded waits have run out: every block leaves,
-    the call reports PDLP_ERR_TIMEOUT, and the next solve in the same form succeeds."""
+    """Block 0 begins only when another block's bounded wait has run out (for its entries, or where the
+    blocks are not coupled for its sums): every block leaves, the call reports PDLP_ERR_TIMEOUT, and
+    the next solve in the same form succeeds."""
     lp = lpgen.set_cover(7, m=2000, n=8000) if name == "cover" else uncoupled(400)
     with pytest.raises(P.PdlpError, match="PDLP_ERR_TIMEOUT"):
         P.pdlp_solve(lp, P.default_params(precision=prec, debug_skip_barrier=1))
@@ -48,10 +49,12 @@ def test_withheld_sums_time_out_and_the_context_survives(P, name, prec):  # noqa
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-def test_late_sums_of_the_last_attempt_still_fail_the_solve(P, prec):  # noqa: F811
-    """With one attempt per check period block 0's late sums complete its own attempt: it leaves as
-    after a success, while the others have left without their part of the iterate."""
-    lp = lpgen.set_cover(7, m=2000, n=8000)
+@pytest.mark.parametrize("name", ["cover", "uncoupled"])
+def test_a_late_block_that_completes_its_attempt_still_fails_the_solve(P, name, prec):  # noqa: F811
+    """With one attempt per check period the late block 0 finds all that it needs where the blocks
+    are not coupled, and leaves as after a success, while the others have left without their part
+    of the iterate."""
+    lp = lpgen.set_cover(7, m=2000, n=8000) if name == "cover" else uncoupled(400)
     kw = dict(precision=prec, adaptive_step=0, check_period=1)
     with pytest.raises(P.PdlpError, match="PDLP_ERR_TIMEOUT"):
         P.pdlp_solve(lp, P.default_params(debug_skip_barrier=1, iter_limit=50, **kw))
