@@ -355,9 +355,11 @@ __global__ void __launch_bounds__(NB, 6) k_gnn_spmm(int rows, const int* __restr
 // Measured with the LP of 100,000 columns (cold, ncu): a forward layer 62.8 us with float32
 // multiply-adds, 25 without the remainder (relative error of a gradient against float64 1.3e-7
 // instead of 5e-8: not kept), 34.5 as here (5.0e-8; the predictions' 3.8e-8 / 5.1e-8 before
-// 4.6e-8 / 5.6e-8); 50,000 columns backward 58.9 -> 45.3 us.  What bounds it is the issue of the
-// warp-level mma.sync (one in about 24 cycles per SM quarter at every mix tried).  tcgen05.mma is
-// not used: the remainder needs the accumulator in registers and negated after every 16 terms.
+// 4.6e-8 / 5.6e-8); backward 84.6 us, and of 50,000 columns 58.9 -> 45.3 with six of its nine
+// products.  What bounds it are chains of dependent mma.sync at under four warps per scheduler (ncu:
+// the tensor pipe 40 % active forward and 48 % backward, an instruction issued in 52 and 40 % of the
+// cycles, DRAM below 20 %).  tcgen05.mma is not used: the remainder needs the accumulator in
+// registers and negated after every 16 terms.
 using u32 = unsigned;
 
 // the pieces of (a, b), packed two to a word; an infinity is all in the first piece
@@ -799,7 +801,7 @@ struct Sum3 {
 // each add every 32nd partial of them (one 128-byte line per warp and partial), then one warp adds
 // the 32 sums in order.  In float64 the conversions and additions held that pipe (2.5 million of
 // each for the 304 partials of a dense layer); the float32 triples cost thirteen additions of the
-// other pipe and are no less accurate.  A sum that leaves their range (or is undefined) is added up
+// other pipe and are no less accurate (a dense layer's partials: 10.5 us cold).  A sum that leaves their range (or is undefined) is added up
 // again in float64.
 constexpr int kReduceNB = 1024;
 __global__ void __launch_bounds__(kReduceNB) k_gnn_reduce(const float* __restrict__ part, int nblk,

@@ -29,8 +29,8 @@
 // done; y alternates between two buffers, and so do the posted sums (res_slot).
 // Every wait is bounded as in the cooperative kernel of iter_kernels.cuh.
 //
-// Measured per attempt on a GB300 (three launches -> here): see the table at auto_form() in
-// solver.cu, which chooses the form.
+// Measured per attempt on a GB300: see the table above one_block_nnz() in solver.cu, where the form
+// is chosen.
 #pragma once
 
 #include "internal.h"

@@ -551,7 +551,7 @@ struct SetupOut {
 //   covering 10,000 x 40,000       269,989     14.2 / 13.3                        5.4
 //   covering 50,000 x 200,000    1,350,409     22.3 / 20.3                 18.5 / 12.5
 //   energy system, 24 h             21,600     21.1                         4.5
-//   energy system, 720 h           648,000     18.8                  9.9 to 11.6
+//   energy system, 720 h           648,000     18.8                 10.2 or 12.7 (by its lines' graph)
 // and in float64 (the one block's chains of float64 operations are about as long as the exchange):
 //   relaxation 40 x 80                 320     15.5             4.1           5.0
 //   covering 40 x 160                1,087                      5.2           6.0
